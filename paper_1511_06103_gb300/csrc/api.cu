@@ -40,7 +40,7 @@ struct crf_s {
     // fully connected model
     bool dense = false;
     int N = 0;                   // variables per instance
-    float *K32 = nullptr;        // [B][N][N]
+    float *K32 = nullptr;        // [B][N][dense_k32_pitch(N)]
     __nv_bfloat16 *K16 = nullptr;  // [B][tiles][chunks][128 x 64] swizzled blocks (tensor-core form)
     float *q32[2] = {nullptr, nullptr};            // [B][N][LP] + padding
     __nv_bfloat16 *qt16[2] = {nullptr, nullptr};   // [B][32][N]
@@ -340,17 +340,10 @@ cudaError_t launch_step(crf_t h, const float *eta, int t, int update, double rel
         if (!update || rel_tol <= 0) a.done = nullptr;
         const bool tc = h->bf16 && update && !fp32;
         if (pending) {
-            // the tensor-core step defers its free energy (one partial per row tile)
-            const int d = tc ? 1 : 0;
-            if (*pending && !d) {
-                const cudaError_t e = launch_dense_f_flush(a, t - 1, h->st);
-                if (e != cudaSuccess) return e;
-                if (flushes) ++*flushes;
-                *pending = 0;
-            }
-            a.defer = d;
+            // both forms leave their free energy to the next step
+            a.defer = tc ? dense_tc_tiles(h->N) : dense_f32_parts(h->N, h->L);
             a.prev_pending = *pending;
-            *pending = d;
+            *pending = a.defer;
         }
         if (tc) return launch_dense_step_tc(a, h->tcb, h->st);
         return launch_dense_step_f32(a, h->st);
@@ -600,7 +593,6 @@ crf_status crf_create(const crf_desc *desc, crf_t *out) {
     h->N = h->H * h->W;
     if (dense) {
         h->nd = 0;
-        h->nblk = dense_nblk(h->N);
     }
     h->sparse = sparse;
     if (sparse) {
@@ -622,7 +614,7 @@ crf_status crf_create(const crf_desc *desc, crf_t *out) {
     }
     if (dense) {
         const size_t qn = n_padded(h) + 64 * (size_t)h->LP;   // rows past N read as zero
-        ok = ok && dalloc(&h->K32, (size_t)h->B * h->N * h->N) == cudaSuccess;
+        ok = ok && dalloc(&h->K32, (size_t)h->B * h->N * dense_k32_pitch(h->N)) == cudaSuccess;
         ok = ok && dalloc(&h->q32[0], qn) == cudaSuccess;
         ok = ok && dalloc(&h->q32[1], qn) == cudaSuccess;
         ok = ok && dalloc(&h->feats, (size_t)h->B * h->N * 5) == cudaSuccess;
@@ -662,7 +654,8 @@ crf_status crf_create(const crf_desc *desc, crf_t *out) {
     ok = ok && dalloc(&h->adapt_d, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->eta_auto, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->Lambda, h->B) == cudaSuccess;
-    ok = ok && dalloc(&h->partial, 2 * (size_t)kMaxFParts * h->B * h->nblk) == cudaSuccess;
+    ok = ok && dalloc(&h->partial, 2 * (size_t)h->B * (dense ? dense_f_pitch(h->N) : (size_t)kMaxFParts * h->nblk)) ==
+                   cudaSuccess;
     ok = ok && dalloc(&h->counter, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->fcur, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->done, h->B) == cudaSuccess;
@@ -1034,7 +1027,7 @@ crf_status mf_iterate(crf_t h, const mf_params *p, int32_t *iters_done) {
             if (h->dense) {
                 DenseStepLaunch a = dense_args(h, eta, nsteps - 1, 1, p->rel_tol);
                 if (p->rel_tol <= 0) a.done = nullptr;
-                e = launch_dense_f_flush(a, nsteps - 1, h->st);
+                e = launch_dense_f_flush(a, nsteps - 1, pending, h->st);
             } else {
                 GridStepLaunch a = step_args(h, eta, nsteps - 1, 1, p->rel_tol);
                 if (p->rel_tol <= 0) a.done = nullptr;

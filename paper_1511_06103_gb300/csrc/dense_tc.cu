@@ -66,61 +66,21 @@ struct DenseTcArgs {
     const float *featsT;     // on-the-fly form: [B][nchunk][6][64] (dense_fly_features), else null
     float *split_part;       // [B][ntiles][kSplit][128][32]
     unsigned *tile_count;    // [B][ntiles]
-    double *partial;         // [B][ntiles]
+    double *partial;         // [2][B][dense_f_pitch(N)]
     unsigned *counter;       // [B]
     double *f_trace, *f_cur;
     int *done, *status;
     int N, Np, L, ntiles, nchunk;
     int t, trace_cap, update;
     double rel_tol;
-    int B, defer, prev_pending;   // deferred free energy (DenseStepLaunch): slots of [B][ntiles]
+    int B, defer, prev_pending;   // deferred free energy (DenseStepLaunch)
 };
-
-// Sum of the n row-tile partials of one instance by the whole block: thread
-// k takes k, k + kThreads, ...; shuffle-down trees; warps in order (the order
-// of the ticket form's last-tile sum, so F is the same bit for bit).
-template <int NT>
-__device__ __forceinline__ double dense_sum_partials(const double *p, int n, double *red) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    double acc = 0.0;
-    for (int k = tid; k < n; k += NT) acc += __ldcg(p + k);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    double F = 0.0;
-    for (int k = 0; k < NT / 32; ++k) F += red[k];
-    __syncthreads();   // red is reused
-    return F;
-}
-
-// F of step t_prev from its deferred partials: trace entry and F_cur (by the
-// writer block) and the stopping rule, evaluated identically by every block
-// that asks.  True when instance b stops after step t_prev.
-template <int NT>
-__device__ __forceinline__ bool dense_deferred_f(const DenseTcArgs &a, int b, int t_prev, bool writer,
-                                                 double *red) {
-    const double F =
-        dense_sum_partials<NT>(a.partial + (size_t)(t_prev & 1) * a.B * a.ntiles + (size_t)b * a.ntiles, a.ntiles, red);
-    bool stop = false;
-    if (a.done != nullptr && a.rel_tol > 0.0 && t_prev > 0 && t_prev - 1 < a.trace_cap) {
-        const double Fp = a.f_trace[(size_t)b * a.trace_cap + t_prev - 1];
-        stop = fabs(F - Fp) <= a.rel_tol * fabs(F);
-    }
-    if (writer && threadIdx.x == 0) {
-        a.f_cur[b] = F;
-        if (!isfinite(F)) atomicExch(a.status, -6);
-        if (t_prev < a.trace_cap) a.f_trace[(size_t)b * a.trace_cap + t_prev] = F;
-        if (stop) a.done[b] = t_prev + 1;
-    }
-    return stop;
-}
 
 __global__ void __launch_bounds__(kThreads) dense_f_flush_kernel(const __grid_constant__ DenseTcArgs a) {
     __shared__ double red[kThreads / 32];
     const int b = blockIdx.x;
     if (a.done != nullptr && a.done[b] != 0) return;   // the step copied a stopped instance: no partials
-    dense_deferred_f<kThreads>(a, b, a.t, true, red);
+    dense_deferred_f<kThreads>(a, b, a.t, a.prev_pending, true, red);
 }
 
 // The tile's rows after the product: the k ranges of a tile meet in global
@@ -180,47 +140,10 @@ __device__ __forceinline__ void dense_tc_tail(const DenseTcArgs &a, float (&S)[3
     for (int off = 16; off > 0; off >>= 1) fd += __shfl_down_sync(0xffffffffu, fd, off);
     if (lane == 0) red[warp] = fd;
     __syncthreads();
-    if (a.defer) {
-        // the next step (or the flush kernel) sums this slot
-        if (tid == 0) {
-            double bs = 0.0;
-            for (int k = 0; k < NT / 32; ++k) bs += red[k];
-            a.partial[(size_t)(a.t & 1) * a.B * a.ntiles + (size_t)b * a.ntiles + tile] = bs;
-        }
-        return;
-    }
-    if (tid == 0) {
-        double bs = 0.0;
+    double bs = 0.0;
+    if (tid == 0)
         for (int k = 0; k < NT / 32; ++k) bs += red[k];
-        a.partial[(size_t)b * a.ntiles + tile] = bs;
-        __threadfence();
-        is_last = atomicAdd(a.counter + b, 1u) == (unsigned)(a.ntiles - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    // last tile of the instance: all threads sum fixed strided subsets of the
-    // partials, then a fixed-shape tree (deterministic)
-    __threadfence();
-    double acc = 0.0;
-    for (int k = tid; k < a.ntiles; k += NT) acc += __ldcg(a.partial + (size_t)b * a.ntiles + k);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    __syncthreads();   // red is reused
-    if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    if (tid != 0) return;
-    double F = 0.0;
-    for (int k = 0; k < NT / 32; ++k) F += red[k];
-    a.f_cur[b] = F;
-    if (!isfinite(F)) atomicExch(a.status, -6);
-    if (a.update) {
-        if (a.t < a.trace_cap) a.f_trace[(size_t)b * a.trace_cap + a.t] = F;
-        if (a.rel_tol > 0.0 && a.t > 0 && a.t - 1 < a.trace_cap && a.done != nullptr) {
-            const double Fp = a.f_trace[(size_t)b * a.trace_cap + a.t - 1];
-            if (fabs(F - Fp) <= a.rel_tol * fabs(F)) a.done[b] = a.t + 1;
-        }
-    }
-    a.counter[b] = 0u;
+    dense_f_finish<NT>(a, b, tile, a.ntiles, bs, red, is_last);
 }
 
 template <int LP>
@@ -288,7 +211,7 @@ dense_step_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     __syncthreads();   // is_second is reused below
     if (!stopped && a.prev_pending) {
         const bool writer = tile == 0 && split == 0;
-        if (writer || (a.done != nullptr && a.rel_tol > 0.0)) stopped = dense_deferred_f<kThreads>(a, b, a.t - 1, writer, red);
+        if (writer || (a.done != nullptr && a.rel_tol > 0.0)) stopped = dense_deferred_f<kThreads>(a, b, a.t - 1, a.prev_pending, writer, red);
     }
     if (stopped) {
         // stopping rule met: carry the state through (split 0 copies)
@@ -478,7 +401,7 @@ dense_fly_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (!stopped && a.prev_pending) {
         const bool writer = tile == 0 && split == 0;
         if (writer || (a.done != nullptr && a.rel_tol > 0.0))
-            stopped = dense_deferred_f<kFlyThreads>(a, b, a.t - 1, writer, red);
+            stopped = dense_deferred_f<kFlyThreads>(a, b, a.t - 1, a.prev_pending, writer, red);
     }
     if (stopped) {
         // stopping rule met: carry the state through (split 0 copies)
@@ -672,7 +595,7 @@ cudaError_t encode_2d(CUtensorMap *map, const void *base, long long rows, int Np
 int dense_tc_tiles(int N) { return (N + kTM - 1) / kTM; }
 int dense_tc_pitch(int N) { return (N + kTK - 1) / kTK * kTK; }
 
-cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, cudaStream_t st) {
+cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, int parts, cudaStream_t st) {
     DenseTcArgs a{};
     a.partial = l.partial;
     a.f_trace = l.f_trace;
@@ -687,6 +610,7 @@ cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, cudaStream_t s
     a.update = 1;
     a.rel_tol = l.rel_tol;
     a.B = l.B;
+    a.prev_pending = parts;
     dense_f_flush_kernel<<<l.B, kThreads, 0, st>>>(a);
     return cudaGetLastError();
 }

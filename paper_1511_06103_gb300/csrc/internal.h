@@ -198,8 +198,8 @@ cudaError_t launch_lambda_to_d(const double *Lambda, float *d, int B, cudaStream
 
 // Fully connected Gaussian model (dense.cu, dense_tc.cu).
 struct DenseStepLaunch {
-    const float *K32;            // [B][N][N] FP32 weights (FP32 form)
-    const __nv_bfloat16 *K16;    // [B][N][N] BF16 weights (tensor-core form)
+    const float *K32;            // [B][N][dense_k32_pitch(N)] FP32 weights (FP32 form)
+    const __nv_bfloat16 *K16;    // BF16 weights in blocks (tensor-core form)
     const float *q_in;           // [B][N][LP] q of the state read
     const __nv_bfloat16 *qt_in;  // [B][32][N] BF16 q, label-major (tensor-core form)
     const float *s_in;           // [B][N][LP]
@@ -211,29 +211,35 @@ struct DenseStepLaunch {
     const float *mu;             // [L][L] device
     const float *featsT;         // tensor-core form computing K in the kernel: [B][nchunk][6][64]
                                  // (launch_dense_fly_features), else null (K16 is read)
-    double *partial;             // [B][dense_nblk(N)]; deferred: two slots of [B][dense_tc_tiles(N)]
+    double *partial;             // [2][B][dense_f_pitch(N)] (slot t & 1 when deferred)
     unsigned *counter;           // [B]
     double *f_trace, *f_cur;
     int *done, *status;
     int B, N, L;
     int t, trace_cap, update;
     double rel_tol;
-    // Deferred free energy of the tensor-core step in a loop (as for the
-    // grid step): defer = 1 stores the row tile's partial in slot t & 1 and
-    // takes no ticket; prev_pending = 1 sums step t - 1's partials first.
+    // Deferred free energy in a loop (as for the grid step): defer = n stores
+    // this launch's n partials per instance in slot t & 1 and takes no ticket;
+    // prev_pending = n sums step t - 1's n partials first.
     int defer, prev_pending;
 };
-// The pending free energy of tensor-core step t (dense_tc.cu).
-cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, cudaStream_t st);
+// The pending free energy of step t, `parts` partials per instance (dense_tc.cu).
+cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, int parts, cudaStream_t st);
 // Prescaled features of the on-the-fly tensor-core form, per chunk of 64
 // columns: sqrt(2) s f_k (k = 0..4; s = sqrt(log2 e / (2 theta^2)) of the
 // position or colour group) and -|s f|^2; columns past N get 0 and -1e30.
 cudaError_t launch_dense_fly_features(const float *feats, float *featsT, int B, int N, double theta_pos,
                                       double theta_rgb, cudaStream_t st);
-int dense_nblk(int N);
-int dense_tc_tiles(int N);
+constexpr int kDenseMaxCluster = 8;   // CTAs that split the k range of a row tile of the FP32 step
+int dense_tc_tiles(int N);   // tiles of 128 rows, of both steps
+// Free-energy partials per instance: space for them, and how many a launch of
+// the FP32 step makes (0 on a CUDA error; the tensor-core step makes one per tile).
+__host__ __device__ inline size_t dense_f_pitch(int N) { return (size_t)((N + 127) / 128) * kDenseMaxCluster; }
+int dense_f32_parts(int N, int L);
+// Row pitch (floats) of the FP32 K: whole 16-byte vectors.
+__host__ __device__ inline int dense_k32_pitch(int N) { return (N + 3) / 4 * 4; }
 int dense_tc_pitch(int N);   // row pitch (elements) of the BF16 K and q^T copies
-// K32 [B][N][N] and/or K16 [B][N][pitch] (padding columns zero)
+// K32 [B][N][dense_k32_pitch(N)] and/or K16 in blocks (padding columns zero)
 cudaError_t launch_dense_kernel_build(const float *feats, float *K32, __nv_bfloat16 *K16, int B, int N,
                                       double theta_pos, double theta_rgb, cudaStream_t st);
 // q = exp(s): FP32 [B][N][LP] and/or BF16 label-major [B][32][pitch]
@@ -253,7 +259,7 @@ cudaError_t launch_mu_tilde_extremes(const float *mu_dev, int L, double *nu, cud
 // eta[b] = 1/(1+max(Lambda,0)) (device, FP32).  Returns CRF status codes.
 struct LipschitzJob {
     const float *w;          // pixel-major weights [B][N][n_dirs]
-    const float *Kdense;     // dense model: FP32 weights [B][N][N] (then H = 1, W = N)
+    const float *Kdense;     // dense model: FP32 weights [B][N][dense_k32_pitch(N)] (then H = 1, W = N)
     const float *mu_host;    // [L][L]
     bool mu_sym;
     int B, L, H, W, P, conn;

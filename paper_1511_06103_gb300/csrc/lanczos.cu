@@ -204,7 +204,7 @@ lz_step_a_dense_kernel(LzState st, const float *__restrict__ K, LzGeom g, int nb
     const int row = blockIdx.x * (kLzThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     double dot = 0.0;
     if (row < N) {
-        const float *kr = K + ((size_t)b * N + row) * N;
+        const float *kr = K + ((size_t)b * N + row) * dense_k32_pitch(N);
         double acc = 0.0;
         for (int j = lane; j < N; j += 32) acc += (double)kr[j] * v[j];
 #pragma unroll

@@ -54,6 +54,21 @@ cudaError_t encode_state(CUtensorMap *m, const float *base, int B, int H, int W,
     return encode_4d(m, base, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, B, H, W, LP, box0, box1, box2);
 }
 
+cudaError_t encode_2d_f32(CUtensorMap *m, const float *base, long long rows, int cols, int pitch, int box_rows,
+                          int box_cols) {
+    const PFN_cuTensorMapEncodeTiled_v12000 enc = encoder();
+    if (enc == nullptr) return cudaErrorNotSupported;
+    if ((reinterpret_cast<uintptr_t>(base) & 15u) != 0u || pitch % 4 != 0) return cudaErrorInvalidValue;
+    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)pitch * 4};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    cuuint32_t estr[2] = {1u, 1u};
+    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t encode_grid_maps(GridTmaMaps *m, const GridStepLaunch &l, int LP, int CS) {
     cudaError_t e = encode_state(&m->s_in, l.s_in, l.B, l.H, l.W, LP, CS, GX + 2, GY + 2);
     if (e == cudaSuccess) e = encode_state(&m->U, l.U, l.B, l.H, l.W, LP, CS, GX, GY);

@@ -12,4 +12,9 @@ namespace proxmf {
 cudaError_t encode_state(CUtensorMap *m, const float *base, int B, int H, int W, int LP, int box0, int box1,
                          int box2);
 
+// [rows][cols] FP32 with a row pitch in floats (a multiple of 4), boxes of
+// box_rows x box_cols; columns past cols and rows past rows are zero-filled.
+cudaError_t encode_2d_f32(CUtensorMap *m, const float *base, long long rows, int cols, int pitch, int box_rows,
+                          int box_cols);
+
 }  // namespace proxmf
