@@ -37,6 +37,7 @@ struct crf_s {
     int *sp_out_ptr = nullptr, *sp_out_col = nullptr, *sp_in_ptr = nullptr, *sp_in_col = nullptr;
     float *sp_out_w = nullptr, *sp_in_w = nullptr;
     double *sp_nu = nullptr;     // [2] extreme eigenvalues of C mu C
+    int sp_split = 1;            // lane groups per adjacency list (sparse_split)
     // fully connected model
     bool dense = false;
     int N = 0;                   // variables per instance
@@ -59,7 +60,7 @@ struct crf_s {
     float gamma1 = 0.f, gamma2 = 0.f, eps = 0.f;
     float *eta_auto = nullptr;   // [B]
     double *Lambda = nullptr;    // [B]
-    double *partial = nullptr;   // [2][B][nblk][kMaxFParts] free-energy partials (two slots: deferred sums)
+    double *partial = nullptr;   // [2][B][f_pitch] free-energy partials (two slots: deferred sums)
     unsigned *counter = nullptr; // [B]
     double *ftrace = nullptr;    // [B][trace_cap]
     double *fcur = nullptr;      // [B]
@@ -162,6 +163,11 @@ crf_status check_handle(crf_t h) {
 size_t n_pix(const crf_t h) { return (size_t)h->B * h->H * h->W; }
 size_t n_rows(const crf_t h) { return n_pix(h) * h->L; }
 size_t n_padded(const crf_t h) { return n_pix(h) * h->LP; }
+// free-energy partials of one instance, in each of the two slots
+size_t f_pitch(const crf_t h) {
+    return h->dense ? dense_f_pitch(h->N)
+                    : (h->sparse ? (size_t)sparse_max_blocks(h->N) : (size_t)kMaxFParts * h->nblk);
+}
 
 void free_all(crf_t h) {
     float *fs[] = {h->U, h->s[0], h->s[1], h->w, h->eta_fixed, h->eta_auto, h->staging, h->adapt_d, h->mom, h->vv};
@@ -193,10 +199,14 @@ void free_all(crf_t h) {
     for (float *p : ad)
         if (p) cudaFree(p);
     for (auto &g : h->graphs) cudaGraphExecDestroy(g.exec);
-    h->graphs.clear();
     if (h->cap_st) cudaStreamDestroy(h->cap_st);
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
+}
+
+void drop_graphs(crf_t h) {
+    for (auto &g : h->graphs) cudaGraphExecDestroy(g.exec);
+    h->graphs.clear();
 }
 
 template <typename T>
@@ -220,8 +230,7 @@ crf_status ensure_trace(crf_t h, int iters) {
     }
     h->ftrace = nt;
     h->trace_cap = cap;
-    for (auto &g : h->graphs) cudaGraphExecDestroy(g.exec);   // they captured the old trace buffer
-    h->graphs.clear();
+    drop_graphs(h);   // they captured the old trace buffer
     return CRF_OK;
 }
 
@@ -327,12 +336,18 @@ cudaError_t launch_step(crf_t h, const float *eta, int t, int update, double rel
         a.N = h->N;
         a.L = h->L;
         a.LP = h->LP;
-        a.nblk = h->nblk;
+        a.fpitch = f_pitch(h);
+        a.split = h->sp_split;
         a.t = t;
         a.trace_cap = h->trace_cap;
         a.update = update;
         a.rel_tol = rel_tol;
         a.sym = h->mu_sym;
+        if (pending) {
+            a.defer = sparse_blocks(h->N, h->L, h->sp_split);
+            a.prev_pending = *pending;
+            *pending = a.defer;
+        }
         return launch_sparse_step(a, h->st);
     }
     if (h->dense) {
@@ -597,7 +612,6 @@ crf_status crf_create(const crf_desc *desc, crf_t *out) {
     h->sparse = sparse;
     if (sparse) {
         h->nd = 0;
-        h->nblk = sparse_blocks(h->N);
         h->conn = 0;
     }
     h->mu.assign((size_t)h->L * h->L, 0.f);
@@ -654,8 +668,7 @@ crf_status crf_create(const crf_desc *desc, crf_t *out) {
     ok = ok && dalloc(&h->adapt_d, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->eta_auto, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->Lambda, h->B) == cudaSuccess;
-    ok = ok && dalloc(&h->partial, 2 * (size_t)h->B * (dense ? dense_f_pitch(h->N) : (size_t)kMaxFParts * h->nblk)) ==
-                   cudaSuccess;
+    ok = ok && dalloc(&h->partial, 2 * (size_t)h->B * f_pitch(h)) == cudaSuccess;
     ok = ok && dalloc(&h->counter, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->fcur, h->B) == cudaSuccess;
     ok = ok && dalloc(&h->done, h->B) == cudaSuccess;
@@ -871,6 +884,7 @@ crf_status crf_set_graph(crf_t h, const float *mu, int64_t n_edges, const int32_
     for (int i = 0; i < h->L; ++i)
         for (int j = i + 1; j < h->L; ++j)
             if (m[(size_t)i * h->L + j] != m[(size_t)j * h->L + i]) sym = false;
+    drop_graphs(h);   // they hold the old adjacency arrays and their split
     std::vector<int> optr, ocol, iptr, icol;
     std::vector<float> ow, iw;
     build_csr(h->N, n_edges, sv.data(), dv.data(), wv.data(), sym, optr, ocol, ow, iptr, icol, iw);
@@ -917,6 +931,7 @@ crf_status crf_set_graph(crf_t h, const float *mu, int64_t n_edges, const int32_
     h->launches += sym ? 2 : 2;
     h->mu = m;
     h->mu_sym = sym;
+    h->sp_split = sparse_split(h->N, h->L, (int64_t)std::max(ocol.size(), icol.size()));
     h->lambda_valid = true;
     h->has_pairwise = true;
     h->fcur_valid = false;
@@ -1024,10 +1039,10 @@ crf_status mf_iterate(crf_t h, const mf_params *p, int32_t *iters_done) {
         }
         if (pending) {
             cudaError_t e;
-            if (h->dense) {
-                DenseStepLaunch a = dense_args(h, eta, nsteps - 1, 1, p->rel_tol);
-                if (p->rel_tol <= 0) a.done = nullptr;
-                e = launch_dense_f_flush(a, nsteps - 1, pending, h->st);
+            if (h->dense || h->sparse) {
+                FDeferred f{h->partial, f_pitch(h), h->ftrace, h->fcur, p->rel_tol > 0 ? h->done : nullptr,
+                            h->status, h->B, h->trace_cap, p->rel_tol};
+                e = launch_f_flush(f, nsteps - 1, pending, h->st);
             } else {
                 GridStepLaunch a = step_args(h, eta, nsteps - 1, 1, p->rel_tol);
                 if (p->rel_tol <= 0) a.done = nullptr;
@@ -1253,10 +1268,7 @@ crf_status mf_dense_on_the_fly(crf_t h, int32_t enable) {
     const crf_status rc = check_handle(h);
     if (rc != CRF_OK) return rc;
     if (!h->dense || !h->bf16) return CRF_E_UNSUPPORTED;
-    if (h->dense_fly != (enable != 0)) {
-        for (auto &g : h->graphs) cudaGraphExecDestroy(g.exec);   // they recorded the other kernel
-        h->graphs.clear();
-    }
+    if (h->dense_fly != (enable != 0)) drop_graphs(h);   // they recorded the other kernel
     h->dense_fly = enable != 0;
     return CRF_OK;
 }

@@ -35,6 +35,7 @@
 
 #include "dense_common.cuh"
 #include "f32x2.cuh"
+#include "f_deferred.cuh"
 #include "internal.h"
 #include "tc_common.cuh"
 #include "tma_maps.h"
@@ -71,7 +72,8 @@ struct DenseF32Args {
     float *s_out, *q_out;
     __nv_bfloat16 *qt_out;   // [B][32][pitch] BF16 copy of q_out (tensor-core form) or null
     const float *eta, *mu;
-    double *partial;         // [2][B][dense_f_pitch(N)]
+    double *partial;         // [2][B][fpitch]
+    size_t fpitch;           // dense_f_pitch(N)
     unsigned *counter;
     double *f_trace, *f_cur;
     int *done, *status;
@@ -179,7 +181,7 @@ dense_step_f32_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     if (!stopped && a.prev_pending) {
         const bool writer = blockIdx.x == 0;
         if (writer || (a.done != nullptr && a.rel_tol > 0.0))
-            stopped = dense_deferred_f<kDT>(a, b, a.t - 1, a.prev_pending, writer, red);
+            stopped = f_deferred<kDT>(a, b, a.t - 1, a.prev_pending, writer, red);
     }
     const int r0 = kTM * rank / nc, r1 = kTM * (rank + 1) / nc;   // the CTA's share of the tile's rows
     if (stopped) {
@@ -311,7 +313,7 @@ dense_step_f32_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     double bs = 0.0;
     if (tid == 0)
         for (int k = 0; k < kNW; ++k) bs += red[k];
-    dense_f_finish<kDT>(a, b, (int)blockIdx.x, (int)gridDim.x, bs, red, is_last);
+    f_finish<kDT>(a, b, (int)blockIdx.x, (int)gridDim.x, bs, red, is_last);
 }
 
 // CTAs per row tile (a cluster): the k range is split so that the launch fills
@@ -396,6 +398,7 @@ cudaError_t launch_dense_step_f32(const DenseStepLaunch &l, cudaStream_t st) {
     a.eta = l.eta;
     a.mu = l.mu;
     a.partial = l.partial;
+    a.fpitch = dense_f_pitch(l.N);
     a.counter = l.counter;
     a.f_trace = l.f_trace;
     a.f_cur = l.f_cur;

@@ -32,6 +32,7 @@
 #include <cstdint>
 
 #include "dense_common.cuh"
+#include "f_deferred.cuh"
 #include "internal.h"
 #include "tc_common.cuh"
 
@@ -66,7 +67,8 @@ struct DenseTcArgs {
     const float *featsT;     // on-the-fly form: [B][nchunk][6][64] (dense_fly_features), else null
     float *split_part;       // [B][ntiles][kSplit][128][32]
     unsigned *tile_count;    // [B][ntiles]
-    double *partial;         // [2][B][dense_f_pitch(N)]
+    double *partial;         // [2][B][fpitch]
+    size_t fpitch;           // dense_f_pitch(N)
     unsigned *counter;       // [B]
     double *f_trace, *f_cur;
     int *done, *status;
@@ -75,13 +77,6 @@ struct DenseTcArgs {
     double rel_tol;
     int B, defer, prev_pending;   // deferred free energy (DenseStepLaunch)
 };
-
-__global__ void __launch_bounds__(kThreads) dense_f_flush_kernel(const __grid_constant__ DenseTcArgs a) {
-    __shared__ double red[kThreads / 32];
-    const int b = blockIdx.x;
-    if (a.done != nullptr && a.done[b] != 0) return;   // the step copied a stopped instance: no partials
-    dense_deferred_f<kThreads>(a, b, a.t, a.prev_pending, true, red);
-}
 
 // The tile's rows after the product: the k ranges of a tile meet in global
 // memory (the last CTA to finish sums them in range order), then the row
@@ -143,7 +138,7 @@ __device__ __forceinline__ void dense_tc_tail(const DenseTcArgs &a, float (&S)[3
     double bs = 0.0;
     if (tid == 0)
         for (int k = 0; k < NT / 32; ++k) bs += red[k];
-    dense_f_finish<NT>(a, b, tile, a.ntiles, bs, red, is_last);
+    f_finish<NT>(a, b, tile, a.ntiles, bs, red, is_last);
 }
 
 template <int LP>
@@ -211,7 +206,7 @@ dense_step_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     __syncthreads();   // is_second is reused below
     if (!stopped && a.prev_pending) {
         const bool writer = tile == 0 && split == 0;
-        if (writer || (a.done != nullptr && a.rel_tol > 0.0)) stopped = dense_deferred_f<kThreads>(a, b, a.t - 1, a.prev_pending, writer, red);
+        if (writer || (a.done != nullptr && a.rel_tol > 0.0)) stopped = f_deferred<kThreads>(a, b, a.t - 1, a.prev_pending, writer, red);
     }
     if (stopped) {
         // stopping rule met: carry the state through (split 0 copies)
@@ -401,7 +396,7 @@ dense_fly_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (!stopped && a.prev_pending) {
         const bool writer = tile == 0 && split == 0;
         if (writer || (a.done != nullptr && a.rel_tol > 0.0))
-            stopped = dense_deferred_f<kFlyThreads>(a, b, a.t - 1, a.prev_pending, writer, red);
+            stopped = f_deferred<kFlyThreads>(a, b, a.t - 1, a.prev_pending, writer, red);
     }
     if (stopped) {
         // stopping rule met: carry the state through (split 0 copies)
@@ -595,26 +590,6 @@ cudaError_t encode_2d(CUtensorMap *map, const void *base, long long rows, int Np
 int dense_tc_tiles(int N) { return (N + kTM - 1) / kTM; }
 int dense_tc_pitch(int N) { return (N + kTK - 1) / kTK * kTK; }
 
-cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, int parts, cudaStream_t st) {
-    DenseTcArgs a{};
-    a.partial = l.partial;
-    a.f_trace = l.f_trace;
-    a.f_cur = l.f_cur;
-    a.done = l.done;
-    a.status = l.status;
-    a.N = l.N;
-    a.L = l.L;
-    a.ntiles = dense_tc_tiles(l.N);
-    a.t = t;
-    a.trace_cap = l.trace_cap;
-    a.update = 1;
-    a.rel_tol = l.rel_tol;
-    a.B = l.B;
-    a.prev_pending = parts;
-    dense_f_flush_kernel<<<l.B, kThreads, 0, st>>>(a);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_dense_step_tc(const DenseStepLaunch &l, const DenseTcBuffers &tb, cudaStream_t st) {
     CUtensorMap tmQ;
     const int Np = dense_tc_pitch(l.N);
@@ -634,6 +609,7 @@ cudaError_t launch_dense_step_tc(const DenseStepLaunch &l, const DenseTcBuffers 
     a.split_part = tb.split_part;
     a.tile_count = tb.tile_count;
     a.partial = l.partial;
+    a.fpitch = dense_f_pitch(l.N);
     a.counter = l.counter;
     a.f_trace = l.f_trace;
     a.f_cur = l.f_cur;

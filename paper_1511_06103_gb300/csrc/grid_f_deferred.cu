@@ -5,6 +5,8 @@
 // its own tile loads are in flight.  After the last such step this kernel
 // takes it: the fixed-order sum of the tile partials, the trace entry, F_cur
 // and the stopping rule, exactly as the next step would have.
+// The fully connected and edge-list steps do the same (f_deferred.cuh).
+#include "f_deferred.cuh"
 #include "grid_step.cuh"
 
 namespace proxmf {
@@ -35,6 +37,19 @@ cudaError_t launch_grid_f_flush(const GridStepLaunch &l, int t, int parts, cudaS
     a.update = 1;
     a.rel_tol = l.rel_tol;
     grid_f_flush_kernel<<<l.B, 128, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) f_flush_kernel(const __grid_constant__ FDeferred f, int t, int n) {
+    __shared__ double red[8];
+    const int b = blockIdx.x;
+    if (f.done != nullptr && f.done[b] != 0) return;   // the step copied a stopped instance: no partials
+    f_deferred<256>(f, b, t, n, true, red);
+}
+
+cudaError_t launch_f_flush(const FDeferred &f, int t, int n, cudaStream_t st) {
+    if (n < 1 || (size_t)n > f.fpitch) return cudaErrorInvalidValue;
+    f_flush_kernel<<<f.B, 256, 0, st>>>(f, t, n);
     return cudaGetLastError();
 }
 

@@ -196,7 +196,20 @@ cudaError_t launch_to_bf16(const float *src, __nv_bfloat16 *dst, long long rows,
 // d[b] = max(Lambda[b], 0) (FP32)
 cudaError_t launch_lambda_to_d(const double *Lambda, float *d, int B, cudaStream_t st);
 
-// Fully connected Gaussian model (dense.cu, dense_tc.cu).
+// The pending free energy of a fully connected or edge-list step, n partials per
+// instance (f_deferred.cuh): trace entry, F_cur and the stopping rule
+// (grid_f_deferred.cu).
+struct FDeferred {
+    double *partial;         // [2][B][fpitch], slot t & 1
+    size_t fpitch;
+    double *f_trace, *f_cur;
+    int *done, *status;
+    int B, trace_cap;
+    double rel_tol;
+};
+cudaError_t launch_f_flush(const FDeferred &f, int t, int n, cudaStream_t st);
+
+// Fully connected Gaussian model (dense.cu, dense_f32.cu, dense_tc.cu).
 struct DenseStepLaunch {
     const float *K32;            // [B][N][dense_k32_pitch(N)] FP32 weights (FP32 form)
     const __nv_bfloat16 *K16;    // BF16 weights in blocks (tensor-core form)
@@ -223,8 +236,6 @@ struct DenseStepLaunch {
     // prev_pending = n sums step t - 1's n partials first.
     int defer, prev_pending;
 };
-// The pending free energy of step t, `parts` partials per instance (dense_tc.cu).
-cudaError_t launch_dense_f_flush(const DenseStepLaunch &l, int t, int parts, cudaStream_t st);
 // Prescaled features of the on-the-fly tensor-core form, per chunk of 64
 // columns: sqrt(2) s f_k (k = 0..4; s = sqrt(log2 e / (2 theta^2)) of the
 // position or colour group) and -|s f|^2; columns past N get 0 and -1e30.
@@ -272,7 +283,7 @@ int estimate_lipschitz_grid(const LipschitzJob &job, cudaStream_t st, int *steps
                             long long *launches_out);
 
 
-// General pairwise graphs (sparse.cu): CSR adjacency, one warp per variable.
+// General pairwise graphs (sparse.cu): CSR adjacency.
 struct SparseStepLaunch {
     const float *s_in;       // [B][N][LP] log q^t
     float *s_out;            // [B][N][LP] log q^{t+1}
@@ -285,16 +296,21 @@ struct SparseStepLaunch {
     const float *in_w;
     const float *mu;         // [L][L] device
     const float *eta;        // [B]
-    double *partial;         // [B][nblk]
+    double *partial;         // [2][B][fpitch] (slot t & 1 when deferred)
+    size_t fpitch;           // sparse_max_blocks(N)
     unsigned *counter;       // [B]
     double *f_trace, *f_cur;
     int *done, *status;
-    int B, N, L, LP, nblk;
+    int B, N, L, LP;
+    int split;               // lanes that share an adjacency list (sparse_split)
     int t, trace_cap, update;
     double rel_tol;
+    int defer, prev_pending; // deferred free energy in a loop, as for the dense steps
     bool sym;
 };
-int sparse_blocks(int N);
+int sparse_split(int N, int L, int64_t entries);   // entries: of the longer of the two adjacency arrays
+int sparse_blocks(int N, int L, int split);        // blocks, and free-energy partials, per instance
+int sparse_max_blocks(int N);
 cudaError_t launch_sparse_step(const SparseStepLaunch &a, cudaStream_t st);
 cudaError_t launch_sparse_degree(const int *ptr, const float *w, int N, unsigned *out_bits, cudaStream_t st);
 

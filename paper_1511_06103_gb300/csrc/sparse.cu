@@ -2,21 +2,38 @@
 // as an edge list (Sec. 2.1, Eq. related:pairwise-mrf with an arbitrary edge
 // set; the DBN-shaped layers of the paper's benchmarks are one instance).
 //
-// One warp per variable, one lane per label (L <= 32): the lanes walk the
-// variable's adjacency list in CSR form and accumulate the weighted
-// neighbour marginals with one coalesced 4*LP-byte read per neighbour (for
-// L <= 8 the lanes split the list instead and reduce in a fixed order), then
+// A variable is served by G lanes, each holding one 16-byte vector of its
+// labels (G = labels / 4 rounded up to a power of two; one lane with a pair for
+// two stored labels), times `split` lanes groups that share its adjacency list
+// in CSR form, so a warp works on 32 / (G split) variables at once.  Every lane
+// reads one vector of a neighbour's q per entry, four entries in flight; the
+// groups' sums meet in a fixed-shape shuffle tree.  Then
 //   m = mu S_out + mu^T S_in      (m = mu S for symmetric mu, S over both
 //                                  directions of every edge),
-// the L x L product with the other lanes' S through warp shuffles, and the
-// log-domain step, renormalisation and free-energy term of Eq.
-// method:update_natural as in the grid step.  q = exp(log q) of the new
-// state is written next to it, so that neighbours read q without
-// recomputing exponentials.  Free-energy partials are FP64 per block and
-// reduced in a fixed order by the last block of each instance.
+// with S handed round through shared memory, and the log-domain step,
+// renormalisation and free-energy term of Eq. method:update_natural as in the
+// grid step.  q = exp(log q) of the new state is written next to it, so that
+// neighbours read q without recomputing exponentials; the own q is recomputed
+// from log q, which is read anyway.
+//
+// What bounds it: the gathers (L2: every entry is a row of q) and, for small
+// graphs, the latency of a launch.  The chain per variable is list bounds ->
+// entries -> rows of q -> product -> softmax.  Random graph, N = 262144, 8
+// entries a variable, L = 21: 71 us a step (shared memory 65 % busy with rows of
+// mu, DRAM 125 MB); with one lane per label, 21 of 32 lanes busy and 63
+// instructions a variable for the product alone, 142 us.  Belief-network
+// layers, N = 12288, 43 entries a variable, L = 2: 6.3 us against 14.4 us with a
+// warp per list, four variables in turn and the blocks' ticket.  Twice, four
+// and fourteen times as many blocks: 72, 78 and 104 us on the random graph; five
+// or six resident blocks of fewer registers: 80 and 83 us.
+// Blocks walk the variables grid-stride, at most kSparseBlocks of them (four
+// per SM, all resident), so that the next step can sum their free-energy partials
+// (f_deferred.cuh) while its lists are in flight.
 #include <cmath>
 
 #include "dfloat.cuh"
+#include "f32x2.cuh"
+#include "f_deferred.cuh"
 #include "internal.h"
 
 namespace proxmf {
@@ -25,191 +42,245 @@ namespace {
 
 constexpr int kSW = 8;               // warps per block
 constexpr int kST = kSW * 32;
-// Variables per warp: more per warp for large graphs (fewer blocks, so fewer
-// FP64 block partials for the last block to sum: FP64 is the narrow pipe of
-// this part), one per warp for small ones (enough warps to fill the SMs).
-__host__ __device__ inline int sparse_vpw(int N) { return N >= 131072 ? 8 : (N >= 8192 ? 4 : 1); }
+constexpr int kSparseBlocks = 4 * 152;
 
-// sum_e w_e q[col_e][lane] over one adjacency list, four entries in flight
-__device__ __forceinline__ float gather(const int *__restrict__ ptr, const int *__restrict__ col,
-                                        const float *__restrict__ wt, const float *__restrict__ q, size_t base,
-                                        int i, int lane, int LP) {
-    const int e0 = ptr[i], e1 = ptr[i + 1];
-    float acc = 0.f;
-    int e = e0;
-    for (; e + 4 <= e1; e += 4) {
-        const int c0 = col[e], c1 = col[e + 1], c2 = col[e + 2], c3 = col[e + 3];
-        const float w0 = wt[e], w1 = wt[e + 1], w2 = wt[e + 2], w3 = wt[e + 3];
-        if (lane < LP) {
-            const float q0 = __ldg(q + (base + c0) * LP + lane), q1 = __ldg(q + (base + c1) * LP + lane);
-            const float q2 = __ldg(q + (base + c2) * LP + lane), q3 = __ldg(q + (base + c3) * LP + lane);
-            acc = fmaf(w0, q0, acc);
-            acc = fmaf(w1, q1, acc);
-            acc = fmaf(w2, q2, acc);
-            acc = fmaf(w3, q3, acc);
+// Lanes per variable and labels per lane.
+template <int LP>
+struct SparseGeom {
+    static constexpr int V = LP == 2 ? 2 : 4;
+    static constexpr int GL = LP / V;                                          // lanes with labels
+    static constexpr int G = GL <= 1 ? 1 : GL <= 2 ? 2 : GL <= 4 ? 4 : 8;      // lanes used
+    static constexpr int ROW = G * V;                                          // padded label count
+};
+inline int sparse_lanes(int LP) { return LP <= 4 ? 1 : LP <= 8 ? 2 : LP <= 16 ? 4 : 8; }
+
+template <int V>
+__device__ __forceinline__ void vload(float (&v)[V], const float *p) {
+    if constexpr (V == 4) {
+        const float4 t = *reinterpret_cast<const float4 *>(p);
+        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    } else {
+        const float2 t = *reinterpret_cast<const float2 *>(p);
+        v[0] = t.x, v[1] = t.y;
+    }
+}
+
+template <int V>
+__device__ __forceinline__ void vstore(float *p, const float (&v)[V]) {
+    if constexpr (V == 4)
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else
+        *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+}
+
+// The lane's labels of sum_e w_e q[col_e] over entries e0 + part, + split, ...
+// of one adjacency list, summed over the variable's lane groups.  q points at
+// the lane's labels of variable 0; lanes past the labels (has = false) add 0.
+template <int LP>
+__device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, int e1, const int *__restrict__ col,
+                                       const float *__restrict__ wt, const float *__restrict__ q, int part, int split,
+                                       bool has) {
+    using Gm = SparseGeom<LP>;
+    constexpr int V = Gm::V;
+#pragma unroll
+    for (int l = 0; l < V; ++l) S[l] = 0.f;
+    int e = e0 + part;
+    for (; e + 3 * split < e1; e += 4 * split) {
+        int c[4];
+        float w[4], v[4][V];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            c[j] = __ldg(col + e + j * split);
+            w[j] = __ldg(wt + e + j * split);
+        }
+        if (has) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) vload<V>(v[j], q + (size_t)c[j] * LP);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int l = 0; l < V; ++l) S[l] = fmaf(w[j], v[j][l], S[l]);
         }
     }
-    for (; e < e1; ++e) {
-        const float qj = lane < LP ? __ldg(q + (base + col[e]) * LP + lane) : 0.f;
-        acc = fmaf(wt[e], qj, acc);
+    if (e < e1) {
+        // up to three more entries, together
+        float w[3], v[3][V];
+        int c[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const bool in = e + j * split < e1;
+            c[j] = in ? __ldg(col + e + j * split) : -1;
+            w[j] = in ? __ldg(wt + e + j * split) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            if (has && c[j] >= 0) vload<V>(v[j], q + (size_t)c[j] * LP);
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            if (has && c[j] >= 0) {
+#pragma unroll
+                for (int l = 0; l < V; ++l) S[l] = fmaf(w[j], v[j][l], S[l]);
+            }
     }
-    return acc;
+    __syncwarp();
+    for (int o = split / 2 * Gm::G; o >= Gm::G; o >>= 1) {
+#pragma unroll
+        for (int l = 0; l < V; ++l) S[l] += __shfl_xor_sync(0xffffffffu, S[l], o);
+    }
 }
 
-// The same sums for few labels (L <= LM): the lanes split the adjacency
-// list instead (lane j takes entries j, j + 32, ...), each keeping the L
-// partial sums, which a fixed-shape tree brings to lane 0 and a broadcast
-// hands to every lane.  Returns lane's own label sum (0 past L).
-template <int LM>
-__device__ __forceinline__ float gather_edges(const int *__restrict__ ptr, const int *__restrict__ col,
-                                              const float *__restrict__ wt, const float *__restrict__ q,
-                                              size_t base, int i, int lane, int L, int LP) {
-    float S[LM];
-#pragma unroll
-    for (int l = 0; l < LM; ++l) S[l] = 0.f;
-    const int e0 = ptr[i], e1 = ptr[i + 1];
-#pragma unroll 4
-    for (int e = e0 + lane; e < e1; e += 32) {
-        const float w = wt[e];
-        const float *qr = q + (base + col[e]) * LP;
-#pragma unroll
-        for (int l = 0; l < LM; ++l)
-            if (l < L) S[l] = fmaf(w, __ldg(qr + l), S[l]);
-    }
-    float mine = 0.f;
-#pragma unroll
-    for (int l = 0; l < LM; ++l) {
-        if (l >= L) break;   // warp-uniform
-        float v = S[l];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        v = __shfl_sync(0xffffffffu, v, 0);
-        if (lane == l) mine = v;
-    }
-    return mine;
-}
-
-// Neighbour sums of variable i for lane's label: label-parallel for many
-// labels, edge-parallel for few (LM > 0).
-template <int LM>
-__device__ __forceinline__ float neighbour_sum(const int *ptr, const int *col, const float *wt, const float *q,
-                                               size_t base, int i, int lane, int L, int LP) {
-    if constexpr (LM > 0)
-        return gather_edges<LM>(ptr, col, wt, q, base, i, lane, L, LP);
-    else
-        return gather(ptr, col, wt, q, base, i, lane, LP);
-}
-
-template <bool SYM, int LM>
-__global__ void __launch_bounds__(kST) sparse_step_kernel(const SparseStepLaunch a) {
+template <int LP, bool SYM>
+__global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __grid_constant__ SparseStepLaunch a) {
+    using Gm = SparseGeom<LP>;
+    constexpr int V = Gm::V, G = Gm::G, ROW = Gm::ROW;
     __shared__ double red[kSW];
-    __shared__ int is_last;
+    __shared__ int is_last, stop_in;
+    __shared__ __align__(16) float mus[(SYM ? 1 : 2) * LP * ROW];   // mu^T (and mu), zero-padded
+    __shared__ __align__(16) float sS[kSW][(SYM ? 1 : 2) * 32 * V];   // the S (and T) of a warp's lanes
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int N = a.N, L = a.L, LP = a.LP;
-    const size_t base = (size_t)b * N;
-    const int vpw = sparse_vpw(N);
-    const int i0 = (blockIdx.x * kSW + warp) * vpw;
+    const int N = a.N, L = a.L, split = a.split;
+    const size_t base = (size_t)b * N * LP;
+    const int g = lane & (G - 1), part = (lane / G) & (split - 1);
+    const int vpw = 32 / (G * split), slot = lane / (G * split);
+    const bool has = g < Gm::GL;
+    const int first = (blockIdx.x * kSW + warp) * vpw, stride = gridDim.x * kSW * vpw;
 
-    if (a.done != nullptr && a.done[b] != 0) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the graph and mu do not change between steps
+    for (int e = threadIdx.x; e < LP * ROW; e += kST) {
+        const int k = e / ROW, l = e - k * ROW;
+        const bool in = k < L && l < L;
+        mus[e] = in ? a.mu[l * L + k] : 0.f;
+        if (!SYM) mus[LP * ROW + e] = in ? a.mu[k * L + l] : 0.f;
+    }
+    int o0 = 0, o1 = 0, i0 = 0, i1 = 0;
+    auto bounds = [&](int i) {
+        if (i >= N) {
+            o0 = o1 = i0 = i1 = 0;
+            return;
+        }
+        o0 = __ldg(a.out_ptr + i);
+        o1 = __ldg(a.out_ptr + i + 1);
+        if (!SYM) {
+            i0 = __ldg(a.in_ptr + i);
+            i1 = __ldg(a.in_ptr + i + 1);
+        }
+    };
+    bounds(first + slot);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // stopped before, or the pending F of the previous step meets the rule:
+    // read once per block (the writer block of this launch may set done[b])
+    if (threadIdx.x == 0) stop_in = a.done != nullptr ? a.done[b] : 0;
+    __syncthreads();
+    bool stopped = stop_in != 0;
+    if (!stopped && a.prev_pending) {
+        const bool writer = blockIdx.x == 0;
+        if (writer || (a.done != nullptr && a.rel_tol > 0.0))
+            stopped = f_deferred<kST>(a, b, a.t - 1, a.prev_pending, writer, red);
+    }
+    if (stopped) {
         // stopping rule met: carry the state through unchanged
-        for (int v = 0; v < vpw; ++v) {
-            const int i = i0 + v;
-            if (a.update && i < N && lane < LP) {
-                const size_t o = (base + i) * LP + lane;
-                a.s_out[o] = a.s_in[o];
-                a.q_out[o] = a.q_in[o];
+        for (int v0 = first; v0 < N; v0 += stride) {
+            const int i = v0 + slot;
+            if (a.update && i < N && has && part == 0) {
+                const size_t o = base + (size_t)i * LP + g * V;
+                float v[V];
+                vload<V>(v, a.s_in + o);
+                vstore<V>(a.s_out + o, v);
+                vload<V>(v, a.q_in + o);
+                vstore<V>(a.q_out + o, v);
             }
         }
         return;
     }
 
-    const bool live = lane < L;
-    __shared__ float mus[kMaxLabels * kMaxLabels];
-    for (int e = threadIdx.x; e < L * L; e += kST) mus[e] = a.mu[e];
-    __syncthreads();
     const float eta = a.eta[b];
+    const float *qb = a.q_in + base + g * V;
     float fh = 0.f, fl = 0.f;   // compensated sum of this lane's F terms
-    for (int v = 0; v < vpw; ++v) {
-        const int i = i0 + v;
-        if (i >= N) break;
-        const size_t o = (base + i) * LP + lane;
-        // a1: neighbour sums and m_l = sum_k mu[l][k] S_k (+ sum_k mu[k][l] T_k)
-        const float S = neighbour_sum<LM>(a.out_ptr, a.out_col, a.out_w, a.q_in, base, i, lane, L, LP);
-        float m = 0.f;
-        if constexpr (SYM) {
-            for (int k = 0; k < L; ++k) {
-                const float Sk = __shfl_sync(0xffffffffu, S, k);
-                if (live) m = fmaf(mus[lane * L + k], Sk, m);
-            }
-        } else {
-            const float T = neighbour_sum<LM>(a.in_ptr, a.in_col, a.in_w, a.q_in, base, i, lane, L, LP);
-            for (int k = 0; k < L; ++k) {
-                const float Sk = __shfl_sync(0xffffffffu, S, k);
-                const float Tk = __shfl_sync(0xffffffffu, T, k);
-                if (live) m = fmaf(mus[lane * L + k], Sk, fmaf(mus[k * L + lane], Tk, m));
+    for (int v0 = first; v0 < N; v0 += stride) {
+        const int i = v0 + slot;
+        const bool act = i < N;
+        const size_t o = base + (size_t)(act ? i : 0) * LP + (has ? g * V : 0);
+        float s[V], u[V];
+        vload<V>(s, a.s_in + o);
+        vload<V>(u, a.U + o);
+        // a1: neighbour sums
+        float S[V], T[V];
+        gather<LP>(S, o0, o1, a.out_col, a.out_w, qb, part, split, has);
+        if (!SYM) gather<LP>(T, i0, i1, a.in_col, a.in_w, qb, part, split, has);
+        bounds(i + stride);   // of the next variable
+        // m_l = sum_k mu[l][k] S_k (+ sum_k mu[k][l] T_k), S through the warp's rows
+        vstore<V>(&sS[warp][lane * V], S);
+        if (!SYM) vstore<V>(&sS[warp][32 * V + lane * V], T);
+        __syncwarp();
+        float2 m[V / 2];
+#pragma unroll
+        for (int l = 0; l < V / 2; ++l) m[l] = splat2(0.f);
+        const float *row = &sS[warp][(lane & ~(G - 1)) * V];
+#pragma unroll
+        for (int h = 0; h < (SYM ? 1 : 2); ++h) {
+#pragma unroll
+            for (int k = 0; k < LP; k += V) {
+                float sk[V];
+                vload<V>(sk, row + h * 32 * V + k);
+#pragma unroll
+                for (int j = 0; j < V; ++j) {
+                    float mk[V];
+                    vload<V>(mk, mus + (h * LP + k + j) * ROW + g * V);
+#pragma unroll
+                    for (int l = 0; l < V / 2; ++l)
+                        m[l] = fma2(make_float2(mk[2 * l], mk[2 * l + 1]), splat2(sk[j]), m[l]);
+                }
             }
         }
+        __syncwarp();   // the rows are overwritten by the next variable
         // a2-a4
-        const float s = live ? a.s_in[o] : 0.f;
-        const float u = live ? a.U[o] : 0.f;
-        const float q = live ? a.q_in[o] : 0.f;
-        {
+        float av[V], fp = 0.f, mx = -INFINITY;
+#pragma unroll
+        for (int l = 0; l < V; ++l) {
+            const bool live = g * V + l < L;
+            const float ml = (l & 1) ? m[l / 2].y : m[l / 2].x;
+            if (live) fp = fmaf(__expf(s[l]), u[l] + 0.5f * ml + s[l], fp);
+            av[l] = live ? fmaf(-eta, u[l] + ml, (1.f - eta) * s[l]) : -INFINITY;
+            mx = fmaxf(mx, av[l]);
+        }
+        if (act && part == 0) {
             float se, ee;
-            two_sum(fh, live ? q * (u + 0.5f * m + s) : 0.f, se, ee);
+            two_sum(fh, fp, se, ee);
             fh = se;
             fl = __fadd_rn(fl, ee);
         }
-        const float av = live ? fmaf(-eta, u + m, (1.f - eta) * s) : -INFINITY;
-        float mx = av;
 #pragma unroll
-        for (int w = 16; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-        float z = live ? __expf(av - mx) : 0.f;
+        for (int w = G / 2; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+        float z = 0.f;
 #pragma unroll
-        for (int w = 16; w > 0; w >>= 1) z += __shfl_xor_sync(0xffffffffu, z, w);
-        const float sn = av - mx - __logf(z);
-        if (a.update && lane < LP) {
-            a.s_out[o] = live ? sn : kPadLogQ;
-            a.q_out[o] = live ? __expf(sn) : 0.f;
+        for (int l = 0; l < V; ++l) z += g * V + l < L ? __expf(av[l] - mx) : 0.f;
+#pragma unroll
+        for (int w = G / 2; w > 0; w >>= 1) z += __shfl_xor_sync(0xffffffffu, z, w);
+        const float lz = mx + __logf(z);
+        if (a.update && act && has && part == 0) {
+            float q[V];
+#pragma unroll
+            for (int l = 0; l < V; ++l) {
+                const bool live = g * V + l < L;
+                s[l] = live ? av[l] - lz : kPadLogQ;
+                q[l] = live ? __expf(s[l]) : 0.f;
+            }
+            vstore<V>(a.s_out + o, s);
+            vstore<V>(a.q_out + o, q);
         }
     }
-    // a5: F partial of the block, FP64, fixed order
-    // double-float warp tree (FP64 is the narrow pipe), one FP64 value per warp
+    // a5: F partial of the block in a fixed order: double-float warp trees (FP64
+    // is the narrow pipe of this part), one FP64 value per warp
     const df fw = warp_sum_df(df_fast_two_sum(fh, fl));
     if (lane == 0) red[warp] = df_to(fw);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double bs = 0.0;
+    double bs = 0.0;
+    if (threadIdx.x == 0)
         for (int k = 0; k < kSW; ++k) bs += red[k];
-        a.partial[(size_t)b * a.nblk + blockIdx.x] = bs;
-        __threadfence();
-        is_last = atomicAdd(a.counter + b, 1u) == (unsigned)(a.nblk - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    // last block of the instance: all threads reduce the partials, each a
-    // fixed strided subset, then a fixed-shape tree
-    __threadfence();
-    double acc = 0.0;
-    for (int k = threadIdx.x; k < a.nblk; k += kST) acc += __ldcg(a.partial + (size_t)b * a.nblk + k);
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, w);
-    __syncthreads();   // red is reused
-    if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    double F = 0.0;
-    for (int k = 0; k < kSW; ++k) F += red[k];
-    a.f_cur[b] = F;
-    if (!isfinite(F)) atomicExch(a.status, -6);
-    if (a.update) {
-        if (a.t < a.trace_cap) a.f_trace[(size_t)b * a.trace_cap + a.t] = F;
-        if (a.rel_tol > 0.0 && a.t > 0 && a.t - 1 < a.trace_cap && a.done != nullptr) {
-            const double Fp = a.f_trace[(size_t)b * a.trace_cap + a.t - 1];
-            if (fabs(F - Fp) <= a.rel_tol * fabs(F)) a.done[b] = a.t + 1;
-        }
-    }
-    a.counter[b] = 0u;
+    f_finish<kST>(a, b, (int)blockIdx.x, (int)gridDim.x, bs, red, is_last);
 }
 
 // max over variables of the summed |w| of the adjacency lists (for the
@@ -225,25 +296,57 @@ __global__ void sparse_degree_kernel(const int *ptr, const float *w, int N, unsi
     if ((threadIdx.x & 31) == 0) atomicMax(out_bits, __float_as_uint(best));
 }
 
+template <int LP>
+cudaError_t launch_lp(const SparseStepLaunch &a, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(sparse_blocks(a.N, a.L, a.split), a.B, 1);
+    cfg.blockDim = dim3(kST, 1, 1);
+    cfg.stream = st;
+    // programmatic dependent launch: mu and the first list bounds are read
+    // while the previous step drains
+    cudaLaunchAttribute pdl[1];
+    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = pdl;
+    cfg.numAttrs = 1;
+    return a.sym ? cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, true>, a)
+                 : cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, false>, a);
+}
+
 }  // namespace
 
-int sparse_blocks(int N) { return (N + kSW * sparse_vpw(N) - 1) / (kSW * sparse_vpw(N)); }
+// Lane groups per adjacency list: as many as it takes to have about 98304
+// threads (20 warps per SM), but no more than half the mean list length, so
+// that a group has at least two entries of its own on average.
+int sparse_split(int N, int L, int64_t entries) {
+    const int lanes = sparse_lanes(storage_labels(L));
+    int split = 1;
+    while (2 * split * lanes <= 32 && (int64_t)N * lanes * split < 98304 && entries >= (int64_t)4 * split * N)
+        split *= 2;
+    return split;
+}
+
+int sparse_blocks(int N, int L, int split) {
+    const int per = kSW * 32 / (sparse_lanes(storage_labels(L)) * split);
+    return std::min((N + per - 1) / per, kSparseBlocks);
+}
+
+int sparse_max_blocks(int N) { return std::min((N + kSW - 1) / kSW, kSparseBlocks); }
 
 cudaError_t launch_sparse_step(const SparseStepLaunch &a, cudaStream_t st) {
-    dim3 grid(sparse_blocks(a.N), a.B);
-    // up to 8 labels the lanes split the adjacency lists instead of the labels
-    if (a.L <= 8) {
-        if (a.sym)
-            sparse_step_kernel<true, 8><<<grid, kST, 0, st>>>(a);
-        else
-            sparse_step_kernel<false, 8><<<grid, kST, 0, st>>>(a);
-    } else {
-        if (a.sym)
-            sparse_step_kernel<true, 0><<<grid, kST, 0, st>>>(a);
-        else
-            sparse_step_kernel<false, 0><<<grid, kST, 0, st>>>(a);
+    if (a.defer && a.defer != sparse_blocks(a.N, a.L, a.split)) return cudaErrorInvalidValue;
+    switch (a.LP) {
+    case 2: return launch_lp<2>(a, st);
+    case 4: return launch_lp<4>(a, st);
+    case 8: return launch_lp<8>(a, st);
+    case 12: return launch_lp<12>(a, st);
+    case 16: return launch_lp<16>(a, st);
+    case 20: return launch_lp<20>(a, st);
+    case 24: return launch_lp<24>(a, st);
+    case 28: return launch_lp<28>(a, st);
+    case 32: return launch_lp<32>(a, st);
+    default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_sparse_degree(const int *ptr, const float *w, int N, unsigned *out_bits, cudaStream_t st) {
