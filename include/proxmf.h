@@ -223,9 +223,10 @@ crf_status mf_profile(crf_t h, int32_t enable);
 crf_status mf_profile_read(crf_t h, double *loop_ms, int32_t *launches);
 
 /* mf_use_resident -- 1 (the default): mf_iterate on a grid handle whose
- * iterates fit in the shared memory of a thread-block cluster (up to 8 CTAs
- * per instance, each holding a slab of rows: 4 x rows x W x L_stored floats
- * <= 200 KB per CTA, L <= 16), FP32 form, fixed rule and at least two steps
+ * pixels fit the threads of a thread-block cluster (up to 8 CTAs per instance,
+ * each holding a slab of rows: at most 4096 pixels a slab for L <= 2, 2048 for
+ * L <= 4, 1024 for L <= 8, 512 for L <= 16, and two iterates of the slab in
+ * 200 KB), FP32 form, fixed rule and at least two steps
  * runs the whole loop in one launch (a cluster barrier between steps) and
  * records it as one launch; 0: one launch per step.  Same traces, stopping
  * rule and final state, up to FP32 rounding.  Returns CRF_E_INVALID for a

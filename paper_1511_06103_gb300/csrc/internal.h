@@ -45,9 +45,6 @@ __host__ __device__ constexpr int tc_k(int LT) { return LT <= 16 ? 16 : 32; }
 __host__ __device__ constexpr int tc_sbo(int KP) { return KP / 8 * 128; }
 constexpr int kTcImageBytes = 2 * 32 * 32 * 2;   // mu and mu^T images at the largest tc_k
 
-// Everything one launch of the grid step needs.  State and unaries are
-// pixel-major [B][N][storage_labels(L)], N = H*W, pixel p = y*W + x; edge
-// weights are [B][N][n_dirs] with zero on edges that leave the image.
 // The whole iteration loop of a small grid instance in one launch, one
 // thread-block cluster per instance with the iterates in shared memory
 // (grid_resident.cu).
@@ -71,6 +68,9 @@ size_t grid_resident_smem(int H, int W, int L, int LP);
 bool grid_resident_fits(int H, int W, int L, int LP);
 cudaError_t launch_grid_resident(const GridResidentLaunch &a, cudaStream_t st);
 
+// Everything one launch of the grid step needs.  State and unaries are
+// pixel-major [B][N][storage_labels(L)], N = H*W, pixel p = y*W + x; edge
+// weights are [B][N][n_dirs] with zero on edges that leave the image.
 struct GridStepLaunch {
     const float *s_in;       // log q^t
     float *s_out;            // log q^{t+1}
