@@ -23,6 +23,7 @@
 // recomputation of the trajectory.  Every gradient is accumulated by the
 // thread or block that owns it (dmu through per-block partials reduced in a
 // fixed order), so results do not depend on scheduling.
+#include <algorithm>
 #include <cmath>
 
 #include "internal.h"
@@ -484,15 +485,36 @@ cudaError_t launch_adj_lt(const AdjointStep &a, cudaStream_t st) {
     return a.mu_sym ? launch_adj<LT, 4, true>(a, st) : launch_adj<LT, 4, false>(a, st);
 }
 
-// Through s^0 = logsoftmax(-U): dU += -(gs - q^0 sum gs).
+// Through s^0 = logsoftmax(-U): dU += -(gs - q^0 sum gs).  A row is held by G
+// lanes, one 16-byte vector each (one thread per row read it three times with a
+// stride of a row: 391 us for 1 M rows of 21 labels, now 68 us).
 template <int LP>
-__global__ void adj_init_kernel(const float *gs, const float *s0, float *dU, long long rows, int L) {
-    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < rows;
-         r += (long long)gridDim.x * blockDim.x) {
-        const size_t o = (size_t)r * LP;
-        float sum = 0.f;
-        for (int l = 0; l < L; ++l) sum += gs[o + l];
-        for (int l = 0; l < L; ++l) dU[o + l] += -(gs[o + l] - __expf(s0[o + l]) * sum);
+__global__ void __launch_bounds__(256)
+adj_init_kernel(const float *__restrict__ gs, const float *__restrict__ s0, float *__restrict__ dU, long long rows,
+                int L) {
+    constexpr int V = LP == 2 ? 2 : 4, GL = LP / V, G = GL <= 1 ? 1 : GL <= 2 ? 2 : GL <= 4 ? 4 : 8;
+    const int g = threadIdx.x & (G - 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const long long row = ((long long)blockIdx.x * 4 + k) * (256 / G) + threadIdx.x / G;
+        const bool act = row < rows && g < GL;
+        const long long o = row * LP + g * V;
+        float v[V], s[V], d[V], sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] = s[j] = d[j] = 0.f;
+        if (act) {
+            vget<V>(gs + o, v);
+            vget<V>(s0 + o, s);
+            vget<V>(dU + o, d);
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j) sum += g * V + j < L ? v[j] : 0.f;
+#pragma unroll
+        for (int w = G / 2; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (g * V + j < L) d[j] += -(v[j] - __expf(s[j]) * sum);
+        if (act) vput<V>(dU + o, d);
     }
 }
 
@@ -512,22 +534,23 @@ __global__ void adj_dmu_reduce_kernel(const float *part, int nblk, int LL, float
     if (threadIdx.x == 0) dmu[e] = (float)red[0];
 }
 
-// [B][N][nd] -> [B][nd][H][W]
-__global__ void adj_dw_out_kernel(const float *dw, float *out, int B, int nd, int H, int W) {
-    const long long n = (long long)B * nd * H * W;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % W);
-        const long long r = i / W;
-        const int y = (int)(r % H);
-        const long long bk = r / H;
-        const int k = (int)(bk % nd);
-        const long long b = bk / nd;
-        out[i] = dw[((size_t)b * H * W + (size_t)y * W + x) * nd + k];
+// [B][N][nd] -> [B][nd][H][W], a thread per pixel
+template <int ND>
+__global__ void __launch_bounds__(256) adj_dw_out_kernel(const float *__restrict__ dw, float *__restrict__ out, size_t N) {
+    const size_t b = blockIdx.y;
+    for (size_t p = (size_t)blockIdx.x * 256 + threadIdx.x; p < N; p += (size_t)gridDim.x * 256) {
+        float v[ND];
+        vget<ND>(dw + (b * N + p) * ND, v);
+#pragma unroll
+        for (int k = 0; k < ND; ++k) out[(b * ND + k) * N + p] = v[k];
     }
 }
 
-inline int nb(long long n, int t) { return (int)std::min<long long>((n + t - 1) / t, 1 << 20); }
+template <int LP>
+void launch_adj_init(const AdjointFinish &a, long long rows, cudaStream_t st) {
+    constexpr int GL = LP <= 4 ? 1 : LP / 4, G = GL <= 1 ? 1 : GL <= 2 ? 2 : GL <= 4 ? 4 : 8, per = 4 * 256 / G;
+    adj_init_kernel<LP><<<(unsigned)((rows + per - 1) / per), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L);
+}
 
 }  // namespace
 
@@ -554,19 +577,23 @@ cudaError_t launch_adjoint_finish(const AdjointFinish &a, cudaStream_t st) {
     const long long rows = (long long)a.B * a.H * a.W;
     const int LP = storage_labels(a.L);
     switch (LP) {
-    case 2: adj_init_kernel<2><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
-    case 4: adj_init_kernel<4><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
-    case 8: adj_init_kernel<8><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
-    case 12: adj_init_kernel<12><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
-    case 16: adj_init_kernel<16><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
-    case 20: adj_init_kernel<20><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
-    case 24: adj_init_kernel<24><<<nb(rows, 256), 256, 0, st>>>(a.gs, a.s0, a.dU, rows, a.L); break;
+    case 2: launch_adj_init<2>(a, rows, st); break;
+    case 4: launch_adj_init<4>(a, rows, st); break;
+    case 8: launch_adj_init<8>(a, rows, st); break;
+    case 12: launch_adj_init<12>(a, rows, st); break;
+    case 16: launch_adj_init<16>(a, rows, st); break;
+    case 20: launch_adj_init<20>(a, rows, st); break;
+    case 24: launch_adj_init<24>(a, rows, st); break;
     default: return cudaErrorInvalidValue;
     }
     adj_dmu_reduce_kernel<<<a.L * a.L, 256, 0, st>>>(a.dmu_part, adjoint_blocks(a.B, a.H, a.W), a.L * a.L,
                                                      a.dmu_out);
-    const int nd = a.conn == 8 ? 4 : 2;
-    adj_dw_out_kernel<<<nb(rows * nd, 256), 256, 0, st>>>(a.dw, a.dw_out, a.B, nd, a.H, a.W);
+    const size_t N = (size_t)a.H * a.W;
+    const dim3 grid((unsigned)std::min<size_t>((N + 255) / 256, 65536), a.B);
+    if (a.conn == 8)
+        adj_dw_out_kernel<4><<<grid, 256, 0, st>>>(a.dw, a.dw_out, N);
+    else
+        adj_dw_out_kernel<2><<<grid, 256, 0, st>>>(a.dw, a.dw_out, N);
     return cudaGetLastError();
 }
 

@@ -732,9 +732,8 @@ crf_status crf_set_unary(crf_t h, const float *U, int is_device) {
             src = h->staging;
         }
     }
-    CK(h, launch_rows_to_padded(src, h->U, (long long)n_pix(h), h->L, h->LP, 0.f, h->st));
-    CK(h, launch_init_logq(h->U, h->s[0], (long long)n_pix(h), h->L, h->LP, h->st));
-    h->launches += 2;
+    CK(h, launch_unary_rows(src, h->U, h->s[0], (long long)n_pix(h), h->L, h->LP, 0.f, h->st));
+    h->launches++;
     if (h->U16) {   // the BF16 form's unaries
         CK(h, launch_to_bf16(h->U, h->U16, (long long)n_pix(h), h->LP, u16_pitch(h->LP), h->st));
         h->launches++;

@@ -178,6 +178,10 @@ cudaError_t launch_grid_f_flush(const GridStepLaunch &l, int t, int parts, cudaS
 enum ConvMode { CONV_COPY = 0, CONV_EXP = 1 };
 cudaError_t launch_rows_to_padded(const float *src, float *dst, long long rows, int L, int LP, float pad,
                                   cudaStream_t st);
+// The unaries of a model: padded rows (pad 0) and, if s is given, also
+// s = log softmax(-U) as launch_init_logq writes it, in one pass.
+cudaError_t launch_unary_rows(const float *src, float *dst, float *s, long long rows, int L, int LP, float pad,
+                              cudaStream_t st);
 cudaError_t launch_padded_to_rows(const float *src, float *dst, long long rows, int L, int LP, int mode,
                                   cudaStream_t st);
 // [B][nd][H][W] -> [B][H*W][nd], zeroing entries whose edge leaves the image.

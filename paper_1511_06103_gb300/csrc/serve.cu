@@ -378,8 +378,7 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     *heta = (float)r.p.eta;
 
     SCK(cudaMemcpyAsync(s->staging, hU, N * r.L * sizeof(float), cudaMemcpyHostToDevice, s->st));
-    SCK(launch_rows_to_padded(s->staging, U, (long long)N, r.L, LP, 0.f, s->st));
-    SCK(launch_init_logq(U, s0, (long long)N, r.L, LP, s->st));
+    SCK(launch_unary_rows(s->staging, U, s0, (long long)N, r.L, LP, 0.f, s->st));
     SCK(cudaMemsetAsync(s1, 0, N * LP * sizeof(float), s->st));
     SCK(cudaMemcpyAsync(s->staging, hw, N * nd * sizeof(float), cudaMemcpyHostToDevice, s->st));
     SCK(launch_weights_to_pixel_major(s->staging, w, 1, nd, r.H, r.W, s->st));
