@@ -377,7 +377,9 @@ constexpr long long kLzWaitCycles = 4000000000ll;   // ~2 s at 2 GHz per barrier
 struct LzCoop {
     unsigned *bar;   // [0] arrivals, [1] generation
     int *abort;      // set once a barrier wait ran out; every later barrier fails
-    double *part;    // [2][B][gx] block partials of alpha_k and |u_{k+1}|^2
+    double *part;    // [2][B][gx] block partials of alpha_k and |u_{k+1}|^2 (strided form)
+    double2 *slots;      // [B][2][gx] block partials of t'.u_k and |u_k|^2 (staged form)
+    unsigned *cnt;       // [B] arrivals (staged form)
     int gx;          // blocks per instance
 };
 
@@ -632,14 +634,45 @@ __device__ __forceinline__ df w_times_staged(const float *__restrict__ ws, const
     return df_fast_two_sum(ah, al);
 }
 
-// Steps k0 .. k1-1 of the scalar form with one grid barrier per step.
-// Block bx of an instance owns the contiguous pixels [ps, pe); with
+// u_{k+1} = c1 t' + c2 u_k + c3 u_{k-1}, compensated.
+__device__ __forceinline__ float2 lanczos_update(df c1, df c2, df c3, df t, float2 u, float2 m) {
+    float rh = 0.f, rl = 0.f;
+    acc_prod(rh, rl, c1, t);
+    acc_prod(rh, rl, c2, df{u.x, u.y});
+    acc_prod(rh, rl, c3, df{m.x, m.y});
+    const df r = df_fast_two_sum(rh, rl);
+    return make_float2(r.h, r.l);
+}
+
+// The exchange of a step between the blocks of one instance: a counter that
+// only grows.  Every block adds one per step, releasing its earlier writes, and
+// waits for nblk * (steps so far) arrivals; there is no last arrival that
+// resets and announces, which is one trip to L2 less.  Run by one thread per
+// block, the block's writes ordered before it by the block barrier.  False once
+// this or another block's wait has run out of its clock budget (the abort word
+// is then set).
+__device__ __forceinline__ bool exchange_arrive_wait(unsigned *cnt, unsigned target, int *abort) {
+    red_add_release(cnt, 1u);
+    const long long t0 = clock64();
+    for (unsigned spin = 1; ld_acquire(cnt) < target; ++spin) {
+        if ((spin & 15u) != 0u) continue;
+        if (*(volatile int *)abort != 0) return false;
+        if (clock64() - t0 > kLzWaitCycles) {
+            atomicExch(abort, 1);
+            return false;
+        }
+    }
+    return true;
+}
+
+// Steps k0 .. k1-1 of the scalar form with one exchange between the blocks of
+// an instance per step.  Block bx owns the contiguous pixels [ps, pe); with
 // R1 = W + 1 every neighbour of a pixel p lies in [p - R1, p + R1].  The
 // block keeps u_k, u_{k-1} and the edge weights in shared memory over
 // [ps - 2 R1, pe + 2 R1) and advances u redundantly on the ring
 // [ps - R1, pe + R1) too, with the same arithmetic as the owning blocks (so
 // the copies agree bit for bit): the next product then needs no other
-// block's new values, and the one barrier of a step serves both the
+// block's new values, and the one exchange of a step serves both the
 // reductions and the visibility of the vectors written one step earlier,
 // from which the outer ring is reloaded.  With the unnormalised u_k,
 // t' = W u_k, one reduction gives alpha_k = t'.u_k / |u_k|^2 and
@@ -647,8 +680,22 @@ __device__ __forceinline__ df w_times_staged(const float *__restrict__ ws, const
 //   u_{k+1} = (t' - alpha_k u_k) / |u_k| - (|u_k| / |u_{k-1}|) u_{k-1}.
 // nrm[k] = |u_k| is recorded at step k; a collapsed |u_k| stops the
 // instance with k rows, as in the other forms.  Warp 0 runs the control
-// path (barrier, fixed-order sums, FP64 scalars); warps 1.. own at most PPT
+// path (exchange, fixed-order sums, FP64 scalars); warps 1.. own at most PPT
 // pixels per thread.
+//
+// The step is a latency chain, not a throughput limit (29 % of issue slots
+// before the two changes below),
+// so the chain is what the form shortens:
+//  - the exchange has no last arrival (exchange_arrive_wait), and is among the
+//    blocks of one instance only;
+//  - the inner ring's t' (two ranges of W + 1 pixels, 59 % more products at
+//    512 x 512) needs only the outer ring, so the workers form it while warp 0
+//    sums the partials and forms the scalars; it waits in the outer-ring
+//    entries of the u_{k-1} stage, which hold nothing until the next step.
+// 375 x 500, 8-connected, 288 steps: 7.1 us a step against 8.4 us with the
+// counter that is reset and announced and the ring's products after the scalars.
+// Tagged 128-bit partials that every block polls in place of the counter: 10.2
+// us (150 blocks reading the same 75 lines hold up the writers).
 constexpr int kCoopWorkers = kCoopThreads - 32;
 
 template <int PPT, int ND>
@@ -657,14 +704,12 @@ lz_chunk_halo_kernel(LzState st, const float *__restrict__ w, LzGeom g, LzCoop c
     extern __shared__ float4 smem4[];
     __shared__ double red[2 * (kCoopThreads / 32)];
     __shared__ float fs[6];   // c1 = 1/|u_k|, c2 = -alpha_k/|u_k|, c3 = -|u_k|/|u_{k-1}| (h, l)
-    __shared__ int flags[2];  // [0] grid barrier outcome, [1] the instance stopped
+    __shared__ int flags[2];  // [0] outcome of the exchange, [1] the instance stopped
     const int b = blockIdx.y, bx = blockIdx.x, tid = threadIdx.x, warp = tid >> 5;
-    const unsigned nblocks = gridDim.x * gridDim.y;
     const int N = g.H * g.W, W = g.W, R1 = g.W + 1;
     const size_t base = (size_t)b * N;
     const float *wb = w + base * ND;
-    double *pa = c.part + (size_t)b * c.gx;
-    double *pb = c.part + ((size_t)g.B + b) * c.gx;
+    double2 *slots = c.slots + (size_t)b * 2 * c.gx;   // [2][gx]
     const size_t ld = (size_t)st.ld;
     const int ps = min(N, bx * chunk), pe = min(N, ps + chunk);
     const int o2 = ps - 2 * R1;                 // pixel of stage index 0 (may be negative)
@@ -675,7 +720,8 @@ lz_chunk_halo_kernel(LzState st, const float *__restrict__ w, LzGeom g, LzCoop c
     const int wt = tid - 32;
     float *ws = reinterpret_cast<float *>(smem4);                               // [S][4] weights
     float2 *su = reinterpret_cast<float2 *>(smem4 + S), *sm = su + S;          // u_k, u_{k-1}
-    bool active = st.stop[b] == 0;
+    // a stopped instance has nothing left to do: its blocks exchange with no one else
+    if (st.stop[b] != 0) return;
     // thread 0: |u_{k-1}|, its reciprocal and alpha_{k-1}
     double n_prev = 0.0, a_prev = 0.0, inv_prev = 0.0;
     if (tid == 0) {
@@ -705,17 +751,15 @@ lz_chunk_halo_kernel(LzState st, const float *__restrict__ w, LzGeom g, LzCoop c
         // t' = W u_k on the own pixels, partials of t'.u_k and |u_k|^2 (workers)
         if (wt >= 0) {
             float dh = 0.f, dl = 0.f, nh = 0.f, nl = 0.f;
-            if (active) {
 #pragma unroll
-                for (int j = 0; j < PPT; ++j) {
-                    const int p = ps + wt + j * kCoopWorkers;
-                    if (p < pe) {
-                        tt[j] = w_times_staged<ND>(ws, su, p - o2, W);
-                        const float2 u2 = su[p - o2];
-                        const df u = {u2.x, u2.y};
-                        acc_prod(dh, dl, tt[j], u);
-                        acc_prod(nh, nl, u, u);
-                    }
+            for (int j = 0; j < PPT; ++j) {
+                const int p = ps + wt + j * kCoopWorkers;
+                if (p < pe) {
+                    tt[j] = w_times_staged<ND>(ws, su, p - o2, W);
+                    const float2 u2 = su[p - o2];
+                    const df u = {u2.x, u2.y};
+                    acc_prod(dh, dl, tt[j], u);
+                    acc_prod(nh, nl, u, u);
                 }
             }
             const df d = warp_sum_df(df_fast_two_sum(dh, dl));
@@ -729,28 +773,32 @@ lz_chunk_halo_kernel(LzState st, const float *__restrict__ w, LzGeom g, LzCoop c
         if (warp == 0) {
             // block partials: the warps' values by a fixed-shape tree
             const int lane = tid;
-            double sd = lane >= 1 && lane < kCoopThreads / 32 ? red[lane] : 0.0;
-            double sn = lane >= 1 && lane < kCoopThreads / 32 ? red[16 + lane] : 0.0;
-            sd = warp_sum(sd);
-            sn = warp_sum(sn);
+            double bd = lane >= 1 && lane < kCoopThreads / 32 ? red[lane] : 0.0;
+            double bn = lane >= 1 && lane < kCoopThreads / 32 ? red[16 + lane] : 0.0;
+            bd = warp_sum(bd);
+            bn = warp_sum(bn);
+            // two rows: a block writes row k & 1 again at step k + 2, after every
+            // block has arrived at step k + 1, that is, has read step k's
+            double2 *row = slots + (size_t)(k & 1) * c.gx;
             if (lane == 0) {
-                __stcg(pa + bx, sd);
-                __stcg(pb + bx, sn);
-                flags[0] = grid_arrive_wait(c, nblocks) ? 1 : 0;
+                __stcg(row + bx, make_double2(bd, bn));
+                flags[0] = exchange_arrive_wait(c.cnt + b, (unsigned)(k + 1) * c.gx, c.abort) ? 1 : 0;
             }
         }
         __syncthreads();
         if (flags[0] == 0) return;
         if (warp == 0) {
             // both sums of the instance in one pass over the partials
+            const double2 *row = slots + (size_t)(k & 1) * c.gx;
             double sd = 0.0, sn = 0.0;
             for (int i = tid; i < c.gx; i += 32) {
-                sd += __ldcg(pa + i);
-                sn += __ldcg(pb + i);
+                const double2 v = __ldcg(row + i);
+                sd += v.x;
+                sn += v.y;
             }
             sd = warp_sum(sd);
             sn = warp_sum(sn);
-            if (tid == 0 && active) {
+            if (tid == 0) {
                 // one reciprocal square root; the rest are products
                 const double inv = rsqrt(sn);
                 const double nk = sn * inv;
@@ -777,42 +825,38 @@ lz_chunk_halo_kernel(LzState st, const float *__restrict__ w, LzGeom g, LzCoop c
                 n_prev = nk;
                 inv_prev = inv;
             }
-        } else if (active) {
+        } else {
             // outer ring of u_k from L2: written by its owners at step k - 1,
-            // visible since this step's barrier
+            // visible since this step's exchange
             for (int q = lo2 + wt; q < lo1; q += kCoopWorkers) su[q - o2] = __ldcg(ucur + q);
             for (int q = hi1 + wt; q < hi2; q += kCoopWorkers) su[q - o2] = __ldcg(ucur + q);
+            asm volatile("bar.sync 1, %0;" ::"n"(kCoopWorkers) : "memory");
+            for (int i = wt; i < nring; i += kCoopWorkers) {
+                const int q = i < nl1 ? lo1 + i : pe + (i - nl1);
+                const df t = w_times_staged<ND>(ws, su, q - o2, W);
+                sm[q - o2 + (i < nl1 ? -R1 : R1)] = make_float2(t.h, t.l);
+            }
         }
         __syncthreads();
-        if (flags[1] != 0) active = false;
+        if (flags[1] != 0) return;
         // u_{k+1} on the own pixels (also to L2) and on the inner ring, into sm
-        if (wt >= 0 && active) {
+        if (wt >= 0) {
             const df c1 = {fs[0], fs[1]}, c2 = {fs[2], fs[3]}, c3 = {fs[4], fs[5]};
 #pragma unroll
             for (int j = 0; j < PPT; ++j) {
                 const int p = ps + wt + j * kCoopWorkers;
                 if (p < pe) {
-                    const float2 u = su[p - o2], m = sm[p - o2];
-                    float rh = 0.f, rl = 0.f;
-                    acc_prod(rh, rl, c1, tt[j]);
-                    acc_prod(rh, rl, c2, df{u.x, u.y});
-                    acc_prod(rh, rl, c3, df{m.x, m.y});
-                    const df r = df_fast_two_sum(rh, rl);
-                    const float2 r2 = make_float2(r.h, r.l);
+                    const float2 r2 = lanczos_update(c1, c2, c3, tt[j], su[p - o2], sm[p - o2]);
                     sm[p - o2] = r2;
                     __stcg(unext + p, r2);
                 }
             }
             for (int i = wt; i < nring; i += kCoopWorkers) {
                 const int q = i < nl1 ? lo1 + i : pe + (i - nl1);
-                const df t = w_times_staged<ND>(ws, su, q - o2, W);
-                const float2 u = su[q - o2], m = sm[q - o2];
-                float rh = 0.f, rl = 0.f;
-                acc_prod(rh, rl, c1, t);
-                acc_prod(rh, rl, c2, df{u.x, u.y});
-                acc_prod(rh, rl, c3, df{m.x, m.y});
-                const df r = df_fast_two_sum(rh, rl);
-                sm[q - o2] = make_float2(r.h, r.l);
+                float2 *park = sm + (q - o2 + (i < nl1 ? -R1 : R1));
+                const float2 t = *park;
+                *park = make_float2(0.f, 0.f);   // entries outside the instance stay zero
+                sm[q - o2] = lanczos_update(c1, c2, c3, df{t.x, t.y}, su[q - o2], sm[q - o2]);
             }
         }
         __syncthreads();
@@ -1247,6 +1291,9 @@ int estimate_lipschitz_grid(const LipschitzJob &job, cudaStream_t st, int *steps
         LZ_CHECK(cudaMallocAsync((void **)&C.part, (size_t)2 * B * C.gx * sizeof(double), st));
         LZ_CHECK(cudaMemsetAsync(C.bar, 0, 2 * sizeof(unsigned), st));
         LZ_CHECK(cudaMemsetAsync(C.abort, 0, sizeof(int), st));
+        LZ_CHECK(cudaMallocAsync((void **)&C.slots, (size_t)2 * B * C.gx * sizeof(double2), st));
+        LZ_CHECK(cudaMallocAsync((void **)&C.cnt, (size_t)B * sizeof(unsigned), st));
+        LZ_CHECK(cudaMemsetAsync(C.cnt, 0, (size_t)B * sizeof(unsigned), st));
     } else {
         // one graph of kChunk steps, captured once and replayed
         LZ_CHECK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
@@ -1336,6 +1383,8 @@ done:
     if (C.bar) cudaFreeAsync(C.bar, st);
     if (C.abort) cudaFreeAsync(C.abort, st);
     if (C.part) cudaFreeAsync(C.part, st);
+    if (C.slots) cudaFreeAsync(C.slots, st);
+    if (C.cnt) cudaFreeAsync(C.cnt, st);
     if (mu_dev) cudaFreeAsync(mu_dev, st);
     return rc;
 }
