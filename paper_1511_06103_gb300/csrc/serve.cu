@@ -80,8 +80,9 @@ private:
     size_t used_ = 0;
 };
 
-// Ring of page-locked host memory: blocks are handed out in FIFO order and
-// come back when the event recorded after their last copy has completed.
+// Ring of page-locked host memory.  Blocks are handed out in FIFO order; a
+// block comes back when the event recorded after its last copy (seal) has
+// completed and, where the host still has to read it (held), release was called.
 class PinnedRing {
 public:
     bool init(size_t size) {
@@ -89,30 +90,23 @@ public:
         return cudaHostAlloc((void **)&base_, size, cudaHostAllocDefault) == cudaSuccess;
     }
     ~PinnedRing() {
-        for (auto &b : live_) cudaEventDestroy(b.ev);
+        for (auto &b : live_)
+            if (b.ev) cudaEventDestroy(b.ev);
         for (cudaEvent_t e : spare_) cudaEventDestroy(e);
         if (base_) cudaFreeHost(base_);
     }
     size_t size() const { return size_; }
-    // A block of `bytes` (256-byte aligned), waiting for the oldest blocks to
-    // be released if the ring is full.  nullptr if it can never fit.
-    unsigned char *acquire(size_t bytes) {
+    // A block of `bytes` (256-byte aligned), or nullptr while there is no room.
+    unsigned char *try_acquire(size_t bytes) {
         bytes = (bytes + 255) / 256 * 256;
-        if (bytes > size_) return nullptr;
-        for (;;) {
-            reclaim(false);
-            size_t off;
-            if (fits(bytes, &off)) {
-                pending_off_ = off;
-                pending_bytes_ = bytes;
-                return base_ + off;
-            }
-            if (live_.empty()) return nullptr;
-            cudaEventSynchronize(live_.front().ev);
-        }
+        reclaim();
+        size_t off;
+        if (!fits(bytes, &off)) return nullptr;
+        live_.push_back({off, bytes, nullptr, false});
+        return base_ + off;
     }
-    // Seal the block handed out last: its copies were issued on st.
-    cudaError_t seal(cudaStream_t st) {
+    // Seal the oldest block without an event: its copies were issued on st.
+    cudaError_t seal(cudaStream_t st, bool held = false, cudaEvent_t *ev = nullptr) {
         cudaEvent_t e = nullptr;
         if (!spare_.empty()) {
             e = spare_.back();
@@ -120,28 +114,42 @@ public:
         } else if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
             return cudaErrorMemoryAllocation;
         }
-        const cudaError_t r = cudaEventRecord(e, st);
-        live_.push_back({pending_off_, pending_bytes_, e});
-        return r;
+        for (auto &b : live_)
+            if (!b.ev) {
+                b.ev = e;
+                b.held = held;
+                break;
+            }
+        if (ev) *ev = e;
+        return cudaEventRecord(e, st);
     }
-    cudaEvent_t last_event() const { return live_.back().ev; }
-    void reclaim(bool all) {
-        while (!live_.empty() && (all || cudaEventQuery(live_.front().ev) == cudaSuccess)) {
-            if (all) cudaEventSynchronize(live_.front().ev);
+    void release(const unsigned char *p) {
+        for (auto &b : live_)
+            if (base_ + b.off == p) b.held = false;
+    }
+    // Wait for the oldest block's copies; false when there is nothing to wait for.
+    bool wait_front() {
+        if (live_.empty() || !live_.front().ev) return false;
+        return cudaEventSynchronize(live_.front().ev) == cudaSuccess;
+    }
+
+private:
+    void reclaim() {
+        while (!live_.empty() && live_.front().ev && !live_.front().held &&
+               cudaEventQuery(live_.front().ev) == cudaSuccess) {
             spare_.push_back(live_.front().ev);
             live_.pop_front();
         }
         (void)cudaGetLastError();   // a query of an unfinished event is not an error
     }
-
-private:
     bool fits(size_t bytes, size_t *off) const {
+        if (bytes > size_) return false;
         if (live_.empty()) {
             *off = 0;
             return true;
         }
         const size_t start = live_.front().off, end = live_.back().off + live_.back().bytes;
-        if (end > start || (end == start && live_.size() == 0)) {
+        if (end > start) {
             if (size_ - end >= bytes) {
                 *off = end;
                 return true;
@@ -161,12 +169,12 @@ private:
     struct Block {
         size_t off, bytes;
         cudaEvent_t ev;
+        bool held;
     };
     unsigned char *base_ = nullptr;
     size_t size_ = 0;
     std::deque<Block> live_;
     std::vector<cudaEvent_t> spare_;
-    size_t pending_off_ = 0, pending_bytes_ = 0;
 };
 
 struct Request {
@@ -348,6 +356,18 @@ crf_status ensure_staging(mf_server_t s, size_t floats) {
     return CRF_OK;
 }
 
+void deliver(mf_server_t s, bool wait);
+
+// A block of the ring, waiting for the oldest ones; results whose copies have
+// landed are delivered first, since their blocks are held until then.
+unsigned char *ring_acquire(mf_server_t s, size_t bytes) {
+    for (;;) {
+        deliver(s, false);
+        if (unsigned char *p = s->ring.try_acquire(bytes)) return p;
+        if (!s->ring.wait_front()) return nullptr;
+    }
+}
+
 // Upload and prepare one admitted request in its pool block and slot.
 crf_status admit(mf_server_t s, Request &r, int si) {
     const SlotLayout l = layout_for(r);
@@ -360,7 +380,7 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     float *w = (float *)(base + l.w), *mu = (float *)(base + l.mu), *eta = (float *)(base + l.eta);
     float2 *pairs = (float2 *)(base + l.pairs);
     // everything the admission uploads, in one page-locked block
-    unsigned char *hb = s->ring.acquire(admit_staging_bytes(r));
+    unsigned char *hb = ring_acquire(s, admit_staging_bytes(r));
     if (!hb) return CRF_E_OOM;
     const size_t npairs = (size_t)2 * LT * mu_pair_slots(LT);
     size_t o = 0;
@@ -437,13 +457,12 @@ crf_status retire(mf_server_t s, Request &r, int si) {
     if (r.q_out) {
         crf_status rc = ensure_staging(s, N * r.L);
         if (rc != CRF_OK) return rc;
-        unsigned char *hb = s->ring.acquire(N * r.L * sizeof(float));
+        unsigned char *hb = ring_acquire(s, N * r.L * sizeof(float));
         if (!hb) return CRF_E_OOM;
         SCK(launch_padded_to_rows(final_s, s->staging, (long long)N, r.L, LP, CONV_EXP, s->st));
         SCK(cudaMemcpyAsync(hb, s->staging, N * r.L * sizeof(float), cudaMemcpyDeviceToHost, s->st));
-        SCK(s->ring.seal(s->st));
+        SCK(s->ring.seal(s->st, true, &r.q_ready));
         r.q_host = hb;
-        r.q_ready = s->ring.last_event();
         r.state = 3;
         s->outgoing.push_back(r.ticket);
     } else {
@@ -469,6 +488,7 @@ void deliver(mf_server_t s, bool wait) {
         else if (cudaEventQuery(r.q_ready) != cudaSuccess)
             break;
         std::memcpy(r.q_out, r.q_host, (size_t)r.H * r.W * r.L * sizeof(float));
+        s->ring.release(r.q_host);
         r.q_host = nullptr;
         r.q_ready = nullptr;
         r.state = 2;
@@ -583,7 +603,6 @@ crf_status mf_server_destroy(mf_server_t s) {
     PROXMF_RANGE("mf_server_destroy");
     if (!s) return CRF_OK;
     cudaStreamSynchronize(s->st);
-    s->ring.reclaim(true);
     if (s->exec) cudaGraphExecDestroy(s->exec);
     if (s->graph) cudaGraphDestroy(s->graph);
     if (s->cap) cudaStreamDestroy(s->cap);
