@@ -9,8 +9,9 @@
 //   2. admits queued requests in arrival order while a slot and pool memory
 //      (first-fit) are free: uploads and converts the data, builds q^0 and
 //      the step size on the device, and enters the slot in the tile table;
-//   3. replays a CUDA graph holding one persistent launch over the tiles of
-//      every running request (serve.cuh), once per requested iteration.
+//   3. replays a CUDA graph holding one persistent launch per group of running
+//      requests, side by side, and the launch that ends the iteration
+//      (serve.cuh), once per requested iteration.
 // Requests therefore join and leave between iterations while the others keep
 // running, and every request's arithmetic is that of a solve on its own.
 //
@@ -33,6 +34,7 @@
 #include "../../include/proxmf.h"
 #include "nvtx_range.h"
 #include "serve.cuh"
+#include "tma_maps.h"
 
 using namespace proxmf;
 
@@ -197,15 +199,17 @@ struct Request {
 
 struct mf_server_s {
     cudaStream_t st = nullptr;
-    cudaStream_t cap = nullptr;
+    cudaStream_t cap = nullptr, cap2 = nullptr;     // capture only
+    cudaEvent_t fork = nullptr, join = nullptr;     // capture only
     size_t budget = 0;
     int max_slots = 0;
     unsigned char *pool_base = nullptr;
     Pool *pool = nullptr;
     PinnedRing ring;
     ServeSlot *d_slots = nullptr;
-    ServeTable *d_table = nullptr;
-    ServeTable *h_table[2] = {nullptr, nullptr};   // page-locked, alternating uploads
+    ServeMaps *d_maps = nullptr;
+    ServeTables *d_table = nullptr;
+    ServeTables *h_table[2] = {nullptr, nullptr};   // page-locked, alternating uploads
     cudaEvent_t table_ev[2] = {nullptr, nullptr};
     int table_buf = 0;
     bool table_dirty = false;
@@ -218,9 +222,10 @@ struct mf_server_s {
     std::deque<uint64_t> outgoing;   // results in flight to q_out, in order
     std::unordered_map<uint64_t, Request> reqs;
     uint64_t next_ticket = 1;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    size_t graph_smem = 0;           // dynamic shared memory the graph's launch was recorded with
+    // recorded iterations by (groups running, shared memory of group 2's launch)
+    std::map<std::pair<int, size_t>, cudaGraphExec_t> graphs;
+    volatile int *h_status = nullptr;   // host-mapped: nonzero once a wait in a launch ran out
+    int *d_status = nullptr;
     bool broken = false;
     int sms = 0;
 };
@@ -244,7 +249,7 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Pool layout of one request (byte offsets from its base).
 struct SlotLayout {
-    size_t U, s0, s1, w, pairs, mu, partial, counter, eta, total;
+    size_t U, s0, s1, w, pairs, mu, partial, eta, total;
 };
 
 SlotLayout layout_for(const Request &r) {
@@ -261,18 +266,19 @@ SlotLayout layout_for(const Request &r) {
     l.pairs = o; o += align256((size_t)2 * LT * mu_pair_slots(LT) * 8);
     l.mu = o; o += align256((size_t)r.L * r.L * 4);
     l.partial = o; o += align256((size_t)nbx * nby * 8);
-    l.counter = o; o += 256;
-    l.eta = o; o += 256;
+    l.eta = o; o += 512;
     l.total = o;
     return l;
 }
 
-// Host bytes an admission stages: U and w rows, mu pairs, mu, eta, the slot.
+constexpr size_t kRequestBytes = (size_t)256 << 20;   // largest request: its inputs, and its result
+
+// Host bytes an admission stages: U and w rows, mu pairs, mu, eta, the slot and its maps.
 size_t admit_staging_bytes(const Request &r) {
     const size_t N = (size_t)r.H * r.W;
     const int LT = kernel_labels(r.L), nd = r.conn == 8 ? 4 : 2;
     return align256(N * r.L * 4) + align256(N * nd * 4) + align256((size_t)2 * LT * mu_pair_slots(LT) * 8) +
-           align256((size_t)r.L * r.L * 4) + 256 + align256(sizeof(ServeSlot));
+           align256((size_t)r.L * r.L * 4) + 256 + align256(sizeof(ServeSlot)) + align256(sizeof(ServeMaps));
 }
 
 // The tile table over every running slot (slot order), into the next
@@ -280,8 +286,8 @@ size_t admit_staging_bytes(const Request &r) {
 crf_status upload_table(mf_server_t s) {
     const int k = s->table_buf;
     SCK(cudaEventSynchronize(s->table_ev[k]));   // the previous upload from this buffer is done
-    ServeTable &t = *s->h_table[k];
-    int n = 0, acc = 0;
+    ServeTables &t = *s->h_table[k];
+    int n[kServeGroups] = {}, acc[kServeGroups] = {};
     for (int si = 0; si < s->max_slots; ++si) {
         const uint64_t tk = (uint64_t)s->slot_ticket[si];
         if (!tk) continue;
@@ -289,58 +295,102 @@ crf_status upload_table(mf_server_t s) {
         if (r.state != 1) continue;
         int nbx, nby;
         grid_tiles(r.H, r.W, &nbx, &nby);
-        t.slots[n] = si;
-        t.prefix[n] = acc;
-        acc += nbx * nby;
-        ++n;
+        const int g = serve_group(kernel_labels(r.L), r.sym);
+        t.g[g].slots[n[g]] = si;
+        t.g[g].prefix[n[g]] = acc[g];
+        acc[g] += nbx * nby;
+        ++n[g];
     }
-    t.count = n;
-    t.prefix[n] = acc;
-    const size_t bytes = offsetof(ServeTable, prefix) + (size_t)(n + 1) * sizeof(int);
-    SCK(cudaMemcpyAsync(s->d_table, &t, bytes, cudaMemcpyHostToDevice, s->st));
+    for (int g = 0; g < kServeGroups; ++g) {
+        t.g[g].count = n[g];
+        t.g[g].prefix[n[g]] = acc[g];
+    }
+    SCK(cudaMemcpyAsync(s->d_table, &t, sizeof(ServeTables), cudaMemcpyHostToDevice, s->st));
     SCK(cudaEventRecord(s->table_ev[k], s->st));
     s->table_buf ^= 1;
     s->table_dirty = false;
     return CRF_OK;
 }
 
-// Dynamic shared memory of the serving launch: the largest class running.
-size_t needed_smem(mf_server_t s) {
+// Groups with a running request (a bit each) and the dynamic shared memory of
+// group 2's launch: its largest label count running.
+std::pair<int, size_t> launch_key(mf_server_t s) {
+    int mask = 0;
     size_t m = 0;
     for (int si = 0; si < s->max_slots; ++si) {
         const uint64_t tk = (uint64_t)s->slot_ticket[si];
         if (!tk) continue;
         const Request &r = s->reqs.at(tk);
-        if (r.state == 1) m = std::max(m, serve_tile_smem(kernel_labels(r.L)));
+        if (r.state != 1) continue;
+        const int LT = kernel_labels(r.L), g = serve_group(LT, r.sym);
+        mask |= 1 << g;
+        if (g == 2) m = std::max(m, serve_tile_smem(LT));
     }
-    return m;
+    return {mask, m};
 }
 
-crf_status capture_graph(mf_server_t s, size_t smem) {
-    if (s->exec) {
-        cudaGraphExecDestroy(s->exec);
-        s->exec = nullptr;
-    }
-    if (s->graph) {
-        cudaGraphDestroy(s->graph);
-        s->graph = nullptr;
-    }
-    // persistent grid: every SM, as many blocks as fit with this shared memory
+// Persistent grid of a group's kernel: every SM, as many blocks as fit.
+template <class K>
+cudaError_t resident_grid(mf_server_t s, K kern, int threads, size_t smem, int *grid) {
     int per_sm = 0;
-    SCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, serve_step_kernel, GT, smem));
-    const int grid = s->sms * std::max(per_sm, 1);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    *grid = s->sms * std::max(per_sm, 1);
+    return e;
+}
+
+// One iteration on the capture streams: the groups side by side (two branches,
+// since no two are ordered), then the launch that ends it.
+cudaError_t record_iteration(mf_server_t s, int mask, size_t smem2) {
+    constexpr size_t smem1 = GridTmaGeom<kServePairLT>::bytes, smem0 = serve_tile_smem(2);
+    int grid = 0;
+    cudaError_t e = cudaEventRecord(s->fork, s->cap);
+    const bool side = (mask & 2) != 0 && (mask & 5) != 0;
+    cudaStream_t other = side ? s->cap2 : s->cap;
+    if (e == cudaSuccess && side) e = cudaStreamWaitEvent(s->cap2, s->fork, 0);
+    if (e == cudaSuccess && (mask & 1)) {
+        e = resident_grid(s, serve_step_kernel<true>, GT, smem0, &grid);
+        serve_step_kernel<true><<<grid, dim3(GX, GY, 1), smem0, other>>>(s->d_slots, &s->d_table->g[0]);
+    }
+    if (e == cudaSuccess && (mask & 4)) {
+        e = resident_grid(s, serve_step_kernel<false>, GT, smem2, &grid);
+        serve_step_kernel<false><<<grid, dim3(GX, GY, 1), smem2, other>>>(s->d_slots, &s->d_table->g[2]);
+    }
+    if (e == cudaSuccess && (mask & 2)) {
+        e = resident_grid(s, serve_pairs_kernel, GT2, smem1, &grid);
+        serve_pairs_kernel<<<grid, dim3(GX, GY / 2, 1), smem1, s->cap>>>(s->d_slots, s->d_maps, &s->d_table->g[1],
+                                                                          s->d_status);
+    }
+    if (e == cudaSuccess && side) {
+        e = cudaEventRecord(s->join, s->cap2);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s->cap, s->join, 0);
+    }
+    serve_finish_kernel<<<s->max_slots, GT, 0, s->cap>>>(s->d_slots, s->d_table, s->d_res);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+crf_status capture_graph(mf_server_t s, const std::pair<int, size_t> &key, cudaGraphExec_t *out) {
+    auto it = s->graphs.find(key);
+    if (it != s->graphs.end()) {
+        *out = it->second;
+        return CRF_OK;
+    }
+    if (s->graphs.size() >= 32) {   // bounded
+        SCK(cudaStreamSynchronize(s->st));
+        for (auto &g : s->graphs) cudaGraphExecDestroy(g.second);
+        s->graphs.clear();
+    }
     SCK(cudaStreamBeginCapture(s->cap, cudaStreamCaptureModeThreadLocal));
-    serve_step_kernel<<<grid, dim3(GX, GY, 1), smem, s->cap>>>(s->d_slots, s->d_table, s->d_res);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = record_iteration(s, key.first, key.second);
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(s->cap, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return srv_cuda(s, e != cudaSuccess ? e : e2);
     }
-    s->graph = g;
-    SCK(cudaGraphInstantiate(&s->exec, s->graph, 0));
-    s->graph_smem = smem;
+    const cudaError_t e3 = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    SCK(e3);
+    s->graphs[key] = *out;
     return CRF_OK;
 }
 
@@ -389,7 +439,8 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     float2 *hp = (float2 *)(hb + o); o += align256(npairs * 8);
     float *hmu = (float *)(hb + o); o += align256((size_t)r.L * r.L * 4);
     float *heta = (float *)(hb + o); o += 256;
-    ServeSlot *hsl = (ServeSlot *)(hb + o);
+    ServeSlot *hsl = (ServeSlot *)(hb + o); o += align256(sizeof(ServeSlot));
+    ServeMaps *hmaps = (ServeMaps *)(hb + o);
     std::memcpy(hU, r.U.data(), N * r.L * sizeof(float));
     std::memcpy(hw, r.w.data(), N * nd * sizeof(float));
     for (size_t i = 0; i < npairs; ++i) hp[i] = make_float2(0.f, 0.f);
@@ -404,7 +455,6 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     SCK(launch_weights_to_pixel_major(s->staging, w, 1, nd, r.H, r.W, s->st));
     SCK(cudaMemcpyAsync(pairs, hp, npairs * sizeof(float2), cudaMemcpyHostToDevice, s->st));
     SCK(cudaMemcpyAsync(mu, hmu, (size_t)r.L * r.L * sizeof(float), cudaMemcpyHostToDevice, s->st));
-    SCK(cudaMemsetAsync(base + l.counter, 0, 256, s->st));
     if (r.p.eta > 0)
         SCK(cudaMemcpyAsync(eta, heta, sizeof(float), cudaMemcpyHostToDevice, s->st));
     else
@@ -420,7 +470,6 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     sl.mu_out = pairs;
     sl.mu_in = pairs + (size_t)LT * mu_pair_slots(LT);
     sl.partial = (double *)(base + l.partial);
-    sl.counter = (unsigned *)(base + l.counter);
     sl.eta = eta;
     sl.L = r.L;
     sl.LT = LT;
@@ -435,6 +484,16 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     sl.it = 0;
     sl.active = r.p.max_iters > 0 ? 1 : 0;
     sl.F_prev = 0.0;
+    if (serve_group(LT, r.sym) == 1) {
+        const int CS = tile_stride(LP);
+        ServeMaps &m = *hmaps;
+        for (int k = 0; k < 2; ++k) {
+            SCK(encode_state(&m.s_in[k], sl.s[k], 1, r.H, r.W, LP, CS, GX + 2, GY + 2));
+            SCK(encode_state(&m.s_out[k], sl.s[k], 1, r.H, r.W, LP, CS, GX, 2));
+        }
+        SCK(encode_state(&m.U, U, 1, r.H, r.W, LP, CS, GX, GY));
+        SCK(cudaMemcpyAsync(s->d_maps + si, hmaps, sizeof(ServeMaps), cudaMemcpyHostToDevice, s->st));
+    }
     s->h_res[si].done = sl.active ? 0 : 1;
     s->h_res[si].iters = 0;
     s->h_res[si].F = 0.0;
@@ -477,6 +536,14 @@ crf_status retire(mf_server_t s, Request &r, int si) {
     r.slot = -1;
     s->table_dirty = true;
     return CRF_OK;
+}
+
+// A wait for a tile's copies ran out in a launch: the server is unusable, as a
+// handle is after a step kernel's timeout.
+crf_status check_status(mf_server_t s) {
+    if (*s->h_status == 0) return CRF_OK;
+    s->broken = true;
+    return CRF_E_TIMEOUT;
 }
 
 // Results whose copy has landed reach q_out (in retirement order).
@@ -572,21 +639,29 @@ crf_status mf_server_create(int64_t budget_bytes, int32_t max_slots, void *strea
     s->sms = sms > 0 ? sms : 148;
     bool ok = cudaMalloc((void **)&s->pool_base, s->budget) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&s->d_slots, sizeof(ServeSlot) * max_slots) == cudaSuccess;
-    ok = ok && cudaMalloc((void **)&s->d_table, sizeof(ServeTable)) == cudaSuccess;
+    ok = ok && cudaMalloc((void **)&s->d_maps, sizeof(ServeMaps) * max_slots) == cudaSuccess;
+    ok = ok && cudaMalloc((void **)&s->d_table, sizeof(ServeTables)) == cudaSuccess;
+    ok = ok && cudaHostAlloc((void **)&s->h_status, sizeof(int), cudaHostAllocMapped) == cudaSuccess;
+    ok = ok && cudaHostGetDevicePointer((void **)&s->d_status, (void *)s->h_status, 0) == cudaSuccess;
+    if (ok) *s->h_status = 0;
     ok = ok && cudaMalloc((void **)&s->d_scratch, 8 * sizeof(double)) == cudaSuccess;
     ok = ok && cudaHostAlloc((void **)&s->h_res, sizeof(ServeResult) * max_slots, cudaHostAllocMapped) == cudaSuccess;
     ok = ok && cudaHostGetDevicePointer((void **)&s->d_res, s->h_res, 0) == cudaSuccess;
     for (int k = 0; k < 2 && ok; ++k) {
-        ok = cudaHostAlloc((void **)&s->h_table[k], sizeof(ServeTable), cudaHostAllocDefault) == cudaSuccess;
+        ok = cudaHostAlloc((void **)&s->h_table[k], sizeof(ServeTables), cudaHostAllocDefault) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&s->table_ev[k], cudaEventDisableTiming) == cudaSuccess;
     }
     // page-locked staging: room for the largest requests several times over
-    ok = ok && s->ring.init((size_t)256 << 20);
+    ok = ok && s->ring.init(kRequestBytes + align256(sizeof(ServeMaps)));
     ok = ok && cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) == cudaSuccess;
-    static SmemOptIn optin;   // up to the largest class's tile memory, once per device
-    ok = ok && smem_optin(optin, serve_step_kernel, serve_tile_smem(kMaxLabels)) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithFlags(&s->cap2, cudaStreamNonBlocking) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) == cudaSuccess;
+    static SmemOptIn optin, optin1;   // up to the largest tile memory, once per device
+    ok = ok && smem_optin(optin, serve_step_kernel<false>, serve_tile_smem(kMaxLabels)) == cudaSuccess;
+    ok = ok && smem_optin(optin1, serve_pairs_kernel, GridTmaGeom<kServePairLT>::bytes) == cudaSuccess;
     if (ok) ok = cudaMemsetAsync(s->d_slots, 0, sizeof(ServeSlot) * max_slots, s->st) == cudaSuccess;
-    if (ok) ok = cudaMemsetAsync(s->d_table, 0, sizeof(ServeTable), s->st) == cudaSuccess;
+    if (ok) ok = cudaMemsetAsync(s->d_table, 0, sizeof(ServeTables), s->st) == cudaSuccess;
     if (ok) ok = cudaStreamSynchronize(s->st) == cudaSuccess;
     if (!ok) {
         (void)cudaGetLastError();
@@ -603,9 +678,13 @@ crf_status mf_server_destroy(mf_server_t s) {
     PROXMF_RANGE("mf_server_destroy");
     if (!s) return CRF_OK;
     cudaStreamSynchronize(s->st);
-    if (s->exec) cudaGraphExecDestroy(s->exec);
-    if (s->graph) cudaGraphDestroy(s->graph);
+    for (auto &g : s->graphs) cudaGraphExecDestroy(g.second);
     if (s->cap) cudaStreamDestroy(s->cap);
+    if (s->cap2) cudaStreamDestroy(s->cap2);
+    if (s->fork) cudaEventDestroy(s->fork);
+    if (s->join) cudaEventDestroy(s->join);
+    if (s->d_maps) cudaFree(s->d_maps);
+    if (s->h_status) cudaFreeHost((void *)s->h_status);
     if (s->pool_base) cudaFree(s->pool_base);
     if (s->d_slots) cudaFree(s->d_slots);
     if (s->d_table) cudaFree(s->d_table);
@@ -652,7 +731,7 @@ crf_status mf_server_submit(mf_server_t s, const crf_desc *d, const float *U, co
     r.q_out = q_out;
     r.bytes = layout_for(r).total;
     if (r.bytes > s->budget) return CRF_E_OOM;
-    if (admit_staging_bytes(r) > s->ring.size() || N * r.L * sizeof(float) > s->ring.size()) return CRF_E_OOM;
+    if (admit_staging_bytes(r) > s->ring.size() || N * r.L * sizeof(float) > kRequestBytes) return CRF_E_OOM;
     *ticket = r.ticket;
     s->queue.push_back(r.ticket);
     s->reqs.emplace(r.ticket, std::move(r));
@@ -663,7 +742,8 @@ crf_status mf_server_step(mf_server_t s, int32_t iters, int32_t *in_flight, int3
     PROXMF_RANGE("mf_server_step");
     if (!s || iters < 0) return CRF_E_INVALID;
     if (s->broken) return CRF_E_STATE;
-    crf_status rc;
+    crf_status rc = check_status(s);
+    if (rc != CRF_OK) return rc;
     deliver(s, false);
     // 1. retire finished slots
     for (int si = 0; si < s->max_slots; ++si) {
@@ -700,16 +780,15 @@ crf_status mf_server_step(mf_server_t s, int32_t iters, int32_t *in_flight, int3
         if (rc != CRF_OK) return rc;
     }
     // 3. iterate every in-flight request: one launch per iteration
-    const size_t smem = needed_smem(s);
+    const std::pair<int, size_t> key = launch_key(s);
     int running = 0;
     for (int si = 0; si < s->max_slots; ++si)
         if (s->slot_ticket[si] && s->reqs.at((uint64_t)s->slot_ticket[si]).state == 1) ++running;
     if (running) {
-        if (!s->exec || smem != s->graph_smem) {
-            rc = capture_graph(s, smem);
-            if (rc != CRF_OK) return rc;
-        }
-        for (int i = 0; i < iters; ++i) SCK(cudaGraphLaunch(s->exec, s->st));
+        cudaGraphExec_t exec = nullptr;
+        rc = capture_graph(s, key, &exec);
+        if (rc != CRF_OK) return rc;
+        for (int i = 0; i < iters; ++i) SCK(cudaGraphLaunch(exec, s->st));
     }
     if (in_flight) *in_flight = running;
     if (queued) *queued = (int)s->queue.size();
@@ -733,6 +812,8 @@ crf_status mf_server_sync(mf_server_t s) {
     if (!s) return CRF_E_INVALID;
     if (s->broken) return CRF_E_STATE;
     SCK(cudaStreamSynchronize(s->st));
+    const crf_status rc = check_status(s);
+    if (rc != CRF_OK) return rc;
     deliver(s, true);
     return CRF_OK;
 }
