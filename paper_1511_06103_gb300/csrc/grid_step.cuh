@@ -934,10 +934,10 @@ cudaError_t launch_grid_step_lt(const GridStepLaunch &l, cudaStream_t st) {
             const cudaError_t e = encode_grid_maps(&maps, l, storage_labels(LT), GridTmaGeom<LT>::CS);
             if (e != cudaSuccess) return e;
             if (l.conn == 8)
-                return l.mu_sym ? launch_grid_tma<LT, 8, true>(maps, a, grid, block, st)
-                                : launch_grid_tma<LT, 8, false>(maps, a, grid, block, st);
-            return l.mu_sym ? launch_grid_tma<LT, 4, true>(maps, a, grid, block, st)
-                            : launch_grid_tma<LT, 4, false>(maps, a, grid, block, st);
+                return l.mu_sym ? launch_grid_tma<LT, 8, true>(maps, a, l.mu_host, grid, block, st)
+                                : launch_grid_tma<LT, 8, false>(maps, a, l.mu_host, grid, block, st);
+            return l.mu_sym ? launch_grid_tma<LT, 4, true>(maps, a, l.mu_host, grid, block, st)
+                            : launch_grid_tma<LT, 4, false>(maps, a, l.mu_host, grid, block, st);
         }
     }
     if (l.conn == 8) {

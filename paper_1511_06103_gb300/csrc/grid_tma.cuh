@@ -391,9 +391,22 @@ __device__ __forceinline__ void acc_regs(float2 (&acc)[NP], const float2 (&v)[NP
 // waits on another at the barrier that follows the conversion.
 constexpr int GT2 = GX * GY / 2;   // threads of the two-pixel tile
 
+// Column pairs of mu for 24 and 28 labels, a parameter of this kernel alone: the
+// shared parameter block stays as small as the launches of few labels need.
+// As constant operands they leave the shared-memory pipe to the gather: four
+// 333 x 479 images of 27 labels, 96 -> 76 us a step.  At 32 labels mu stays in
+// shared memory: ptxas takes minutes for the constant operands there.
+constexpr int kMuWideLT = 28;
+template <int LT>
+struct GridMuWide {
+    static constexpr bool used = LT > kMuParamLT && LT <= kMuWideLT;
+    float2 p[used ? LT * (((LT + 1) / 2 + 1) / 2 * 2) : 1];
+};
+
 template <int LT, int CONN>
 __global__ void __launch_bounds__(GT2, GridTmaGeom<LT>::ctas)
-grid_tma2_step_kernel(const __grid_constant__ GridTmaMaps maps, const __grid_constant__ GridStepArgs a) {
+grid_tma2_step_kernel(const __grid_constant__ GridTmaMaps maps, const __grid_constant__ GridStepArgs a,
+                      const __grid_constant__ GridMuWide<LT> wide) {
     using G = GridTmaGeom<LT>;
     constexpr int LP = G::LP, CS = G::CS, TW = G::QW;
     constexpr int NP = (LT + 1) / 2;
@@ -402,7 +415,7 @@ grid_tma2_step_kernel(const __grid_constant__ GridTmaMaps maps, const __grid_con
     constexpr int HALO = 2 * TW + 2 * GY;             // 84 cells
     constexpr int HPW = (HALO + 3) / 4;               // halo cells per warp
     constexpr bool MASK = (LT == LP);
-    constexpr bool kParamMu = mu_in_params<LT, true, false, 0>();
+    constexpr bool kWide = GridMuWide<LT>::used, kParamMu = kWide || mu_in_params<LT, true, false, 0>();
     static_assert(LP >= 4 && LP % 4 == 0, "cells are whole 16-byte vectors");
     static_assert(HPW <= 32, "one halo cell per lane");
     extern __shared__ __align__(1024) uint8_t tsm[];
@@ -598,7 +611,7 @@ grid_tma2_step_kernel(const __grid_constant__ GridTmaMaps maps, const __grid_con
             m2[k] = splat2(0.f);
         }
         if constexpr (kParamMu)
-            pair_matvec2<LT, NP, NPP>(m1, m2, a.mu_p, S1, S2);
+            pair_matvec2<LT, NP, NPP>(m1, m2, kWide ? wide.p : a.mu_p, S1, S2);
         else
             pair_matvec2<LT, NP, NPP>(m1, m2, mus, S1, S2);
     }
@@ -681,14 +694,10 @@ grid_tma2_step_kernel(const __grid_constant__ GridTmaMaps maps, const __grid_con
 cudaError_t encode_grid_maps(GridTmaMaps *m, const GridStepLaunch &l, int LP, int CS);
 
 template <int LT, int CONN, bool SYM>
-cudaError_t launch_grid_tma(const GridTmaMaps &maps, const GridStepArgs &a, dim3 grid, dim3 block, cudaStream_t st) {
+cudaError_t launch_grid_tma(const GridTmaMaps &maps, const GridStepArgs &a, const float2 *mu_host, dim3 grid,
+                            dim3 block, cudaStream_t st) {
     constexpr int bytes = GridTmaGeom<LT>::bytes;
-    // symmetric mu: two pixels per thread
-    auto kern = SYM ? grid_tma2_step_kernel<LT, CONN> : grid_tma_step_kernel<LT, CONN, SYM>;
-    if (SYM) block = dim3(GX, GY / 2, 1);
     static SmemOptIn optin;   // once per device
-    const cudaError_t attr = smem_optin(optin, kern, bytes);
-    if (attr != cudaSuccess) return attr;
     // programmatic dependent launch: the step may start while the previous
     // kernel on the stream drains (the kernel waits before it reads the state)
     cudaLaunchConfig_t cfg = {};
@@ -701,7 +710,23 @@ cudaError_t launch_grid_tma(const GridTmaMaps &maps, const GridStepArgs &a, dim3
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, maps, a);
+    if constexpr (SYM) {
+        // two pixels per thread
+        auto kern = grid_tma2_step_kernel<LT, CONN>;
+        const cudaError_t attr = smem_optin(optin, kern, bytes);
+        if (attr != cudaSuccess) return attr;
+        GridMuWide<LT> wide;
+        constexpr int n = sizeof(wide.p) / sizeof(wide.p[0]);
+        if (wide.used && !mu_host) return cudaErrorInvalidValue;
+        for (int i = 0; i < n; ++i) wide.p[i] = wide.used ? mu_host[i] : make_float2(0.f, 0.f);
+        cfg.blockDim = dim3(GX, GY / 2, 1);
+        return cudaLaunchKernelEx(&cfg, kern, maps, a, wide);
+    } else {
+        auto kern = grid_tma_step_kernel<LT, CONN, SYM>;
+        const cudaError_t attr = smem_optin(optin, kern, bytes);
+        if (attr != cudaSuccess) return attr;
+        return cudaLaunchKernelEx(&cfg, kern, maps, a);
+    }
 }
 
 }  // namespace proxmf
