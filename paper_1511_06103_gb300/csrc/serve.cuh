@@ -59,7 +59,8 @@ struct ServeTable {
 // every request was bound by the tile's chain of latencies (load, convert,
 // gather, product, ticket).  28 requests of 64 to 512 pixels a side with 2, 8 and
 // 21 labels, 60 iterations, from submission to results: 29.0 -> 19.2 ms, of which
-// the host's copies take 12.
+// the host's copies take 12.  An iteration of the 28 (4600 tiles of group 1, 2300
+// of group 0), one launch after another: 52 us, 14 us and 6 us for the finish.
 constexpr int kServeGroups = 3;
 constexpr int kServePairLT = 21;
 inline int serve_group(int LT, bool sym) { return LT == 2 ? 0 : (sym && LT <= kServePairLT) ? 1 : 2; }
@@ -414,8 +415,8 @@ struct ServePairShared {
 // One 32 x 8 tile whose boxes are in flight on the barrier's phase; requests
 // the next one's as soon as their shared memory is free: log q when the
 // neighbour sums are formed, U when the tile's stores have been read.  The
-// arithmetic is grid_tma2_step_kernel's with mu in shared memory.  False when
-// the wait for the boxes ran out.
+// arithmetic is grid_tma2_step_kernel's with mu in shared memory and c formed
+// from U + log q.  False when the wait for the boxes ran out.
 template <int LT>
 __device__ __forceinline__ bool serve_pair_tile(const ServeSlot &sl, const ServeMaps &mp, int local, ServeWalk &walk,
                                                 ServePairShared &sh, int nxt, uint32_t phase, int *status) {
@@ -463,7 +464,7 @@ __device__ __forceinline__ bool serve_pair_tile(const ServeSlot &sl, const Serve
         }
     }
     const float eta = *sl.eta;
-    const float2 neta = splat2(-eta), ome = splat2(1.f - eta);
+    const float2 neta = splat2(-eta);
     const bool ok = tc::mbar_wait(&sh.bar, phase, status);
 
     // halo cells to q, HPW consecutive ones per warp
@@ -500,9 +501,10 @@ __device__ __forceinline__ bool serve_pair_tile(const ServeSlot &sl, const Serve
 #pragma unroll
         for (int k = 0; k < LP / 2; ++k) {
             const float2 q = exp2v(s[k]);
-            const float2 c = fma2(neta, u[k], mul2(ome, s[k]));
+            const float2 us = add2(u[k], s[k]);
+            const float2 c = fma2(neta, us, s[k]);   // -eta U + (1 - eta) log q, one rounding at log q's size
             if (k < NP) {
-                acc = fma2(q, add2(u[k], s[k]), acc);
+                acc = fma2(q, us, acc);
                 (r == 0 ? q1 : q2)[k] = q;
             }
             s[k] = q;
