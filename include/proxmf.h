@@ -340,8 +340,8 @@ crf_status mf_grid_step_noalloc(int32_t topology, int32_t n_labels, int64_t heig
  * mf_server_step retires finished requests (q copied to the request's q_out,
  * slot and pool memory returned), admits queued requests in arrival order as
  * slots and pool memory allow, and then advances every in-flight request by
- * `iters` proximal steps -- one persistent launch per label class per step,
- * replayed from a CUDA graph.  A request stops after max_iters steps or when
+ * `iters` proximal steps -- one graph launch per step, holding a persistent
+ * kernel for each group of requests in flight.  A request stops after max_iters steps or when
  * |F^t - F^{t-1}| <= rel_tol |F^t| (Sec. 3.1), exactly as mf_iterate would
  * stop it, and its arithmetic does not depend on the other requests.
  * eta <= 0 asks for eta = 1/(1 + D max|nu|) with D the largest weighted degree
