@@ -248,9 +248,11 @@ crf_status mf_dense_on_the_fly(crf_t h, int32_t enable);
  * step-size source, the parity of the state buffers) is seen and replays the
  * graph afterwards, which removes the host launch cost per step (small
  * problems are launch-bound); 0 (default): launches are issued one by one.
- * Graphs hold the handle's device buffers and are dropped when the free-
- * energy trace is regrown or the handle is destroyed.  Results are identical
- * either way. */
+ * Graphs hold the handle's device buffers and, on grids, mu; they are dropped
+ * when the free-energy trace is regrown, when crf_set_pairwise brings another
+ * mu (grids), on crf_set_graph, when mf_dense_on_the_fly changes the form, and
+ * with the handle.  New weights or features under the same mu keep them.
+ * Results are identical either way. */
 crf_status mf_use_graphs(crf_t h, int32_t enable);
 
 /* crf_launch_count -- number of kernels this handle has launched so far. */

@@ -807,6 +807,9 @@ crf_status crf_set_pairwise(crf_t h, const float *mu, const float *w_or_feats, c
         if (!sym) return CRF_E_INVALID;
         return set_pairwise_dense(h, m, w_or_feats, theta, is_device);
     }
+    // a recorded step loop holds the kernels chosen for mu's symmetry and a
+    // symmetric mu of up to 28 labels as launch parameters (weights are read from the handle)
+    if (std::memcmp(h->mu.data(), m.data(), LL * sizeof(float)) != 0) drop_graphs(h);
     const size_t nw = n_pix(h) * h->nd;
     std::vector<float2> pairs;
     build_mu_pairs(m, h->L, h->LT, pairs);

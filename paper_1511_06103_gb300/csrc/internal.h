@@ -80,7 +80,7 @@ struct GridStepLaunch {
     const float2 *mu_out;    // device [LT][NPP] column pairs (see mu_pair_slots)
     const float2 *mu_in;     // device [LT][NPP] row pairs
     const float2 *mu_host;   // host copy of the column pairs (first LT * mu_pair_slots(LT)); required
-                             // for symmetric mu with LT <= 21 (copied into the launch parameters)
+                             // for symmetric mu with LT <= 28 (copied into the launch parameters)
     const uint4 *mu_tc;      // tensor-core form: device BF16 operand images of mu, mu^T
     const __nv_bfloat16 *U16;  // tensor-core form: unaries in BF16, [B][N][u16_pitch(LP)] (may be null)
     bool tc;                 // BF16 tensor-core messages (else FP32)
