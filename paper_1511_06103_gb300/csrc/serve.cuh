@@ -15,6 +15,8 @@
 // Results are published to host-mapped memory.
 #pragma once
 
+#include <cfloat>
+
 #include "grid_step.cuh"
 #include "grid_tma.cuh"
 
@@ -502,7 +504,9 @@ __device__ __forceinline__ bool serve_pair_tile(const ServeSlot &sl, const Serve
         for (int k = 0; k < LP / 2; ++k) {
             const float2 q = exp2v(s[k]);
             const float2 us = add2(u[k], s[k]);
-            const float2 c = fma2(neta, us, s[k]);   // -eta U + (1 - eta) log q, one rounding at log q's size
+            // -eta U + (1 - eta) log q, one rounding at log q's size; a forbidden label
+            // (U = inf, log q = -inf, their sum NaN) stays at -inf: fmaxf drops the NaN
+            const float2 c = fma2(neta, make_float2(fmaxf(us.x, -FLT_MAX), fmaxf(us.y, -FLT_MAX)), s[k]);
             if (k < NP) {
                 acc = fma2(q, us, acc);
                 (r == 0 ? q1 : q2)[k] = q;
