@@ -374,7 +374,9 @@ crf_status mf_server_submit(mf_server_t s, const crf_desc *d, const float *U, co
 crf_status mf_server_step(mf_server_t s, int32_t iters, int32_t *in_flight, int32_t *queued);
 
 /* mf_server_poll -- state of a request: 0 queued, 1 running, 2 done (its q_out
- * written); F is F(q^{K-1}) of its last step and iters the steps it took. */
+ * written); F is F(q^{K-1}) of its last step and iters the steps it took.
+ * CRF_E_TIMEOUT once a wait in a launch has run out, for every request that had
+ * not been delivered by then. */
 crf_status mf_server_poll(mf_server_t s, uint64_t ticket, int32_t *state, double *F, int32_t *iters);
 
 /* mf_server_sync -- wait for the server's stream. */

@@ -502,6 +502,14 @@ crf_status admit(mf_server_t s, Request &r, int si) {
     return CRF_OK;
 }
 
+// A wait for a tile's copies ran out in a launch: the server is unusable, as a
+// handle is after a step kernel's timeout.
+crf_status check_status(mf_server_t s) {
+    if (*s->h_status == 0) return CRF_OK;
+    s->broken = true;
+    return CRF_E_TIMEOUT;
+}
+
 // Queue the copy of q of a retired slot and return its slot and pool block
 // (the stream orders every later use of that memory after the copy).
 crf_status retire(mf_server_t s, Request &r, int si) {
@@ -536,14 +544,6 @@ crf_status retire(mf_server_t s, Request &r, int si) {
     r.slot = -1;
     s->table_dirty = true;
     return CRF_OK;
-}
-
-// A wait for a tile's copies ran out in a launch: the server is unusable, as a
-// handle is after a step kernel's timeout.
-crf_status check_status(mf_server_t s) {
-    if (*s->h_status == 0) return CRF_OK;
-    s->broken = true;
-    return CRF_E_TIMEOUT;
 }
 
 // Results whose copy has landed reach q_out (in retirement order).
@@ -750,7 +750,10 @@ crf_status mf_server_step(mf_server_t s, int32_t iters, int32_t *in_flight, int3
         const uint64_t t = (uint64_t)s->slot_ticket[si];
         if (!t) continue;
         Request &r = s->reqs.at(t);
-        if (r.state == 1 && *(volatile int *)&s->h_res[si].done) {
+        if (r.state != 1) continue;
+        const ServeSlotState state = serve_slot_state(s->h_res[si], s->h_status);
+        if (state == ServeSlotState::timed_out) return check_status(s);
+        if (state == ServeSlotState::finished) {
             rc = retire(s, r, si);
             if (rc != CRF_OK) return rc;
         }
@@ -797,10 +800,14 @@ crf_status mf_server_step(mf_server_t s, int32_t iters, int32_t *in_flight, int3
 
 crf_status mf_server_poll(mf_server_t s, uint64_t ticket, int32_t *state, double *F, int32_t *iters) {
     if (!s) return CRF_E_INVALID;
-    deliver(s, false);
     auto it = s->reqs.find(ticket);
     if (it == s->reqs.end()) return CRF_E_INVALID;
     const Request &r = it->second;
+    const crf_status rc = check_status(s);
+    if (rc == CRF_OK)
+        deliver(s, false);
+    else if (r.state != 2)
+        return rc;   // what was delivered before the timeout stays readable
     if (state) *state = r.state == 3 ? 1 : r.state;
     if (F) *F = r.F;
     if (iters) *iters = r.iters;
@@ -817,5 +824,8 @@ crf_status mf_server_sync(mf_server_t s) {
     deliver(s, true);
     return CRF_OK;
 }
+
+// Not part of the ABI: the word of check_status, which a test sets as a launch would.
+int *proxmf_server_status_word(mf_server_t s) { return const_cast<int *>(s->h_status); }
 
 }  // extern "C"

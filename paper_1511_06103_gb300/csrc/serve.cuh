@@ -19,6 +19,7 @@
 
 #include "grid_step.cuh"
 #include "grid_tma.cuh"
+#include "serve_result.h"
 
 namespace proxmf {
 
@@ -36,12 +37,6 @@ struct ServeSlot {
     int it;                  // steps taken (state parity)
     int active;              // 1 while running
     double F_prev;
-};
-
-struct ServeResult {         // host-mapped
-    int done;                // 1 once retired
-    int iters;
-    double F;                // F of the state before the last step
 };
 
 struct ServeTable {
