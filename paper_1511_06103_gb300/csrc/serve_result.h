@@ -16,10 +16,11 @@ enum class ServeSlotState { running, finished, timed_out };
 // its waits runs out; its tiles are then unwritten, and the launch that ends the
 // iteration may still set `done` from what was there before.  The device writes
 // status before done, so the host reads done first: a finished slot is one that
-// was done with the word still clear.
+// was done with the word still clear.  The load of done acquires: the status word,
+// iters and F are read after it on a host that reorders loads (Arm) too.
 inline ServeSlotState serve_slot_state(const ServeResult &r, const volatile int *status) {
-    if (*static_cast<const volatile int *>(&r.done) == 0) return ServeSlotState::running;
-    return *status != 0 ? ServeSlotState::timed_out : ServeSlotState::finished;
+    if (__atomic_load_n(&r.done, __ATOMIC_ACQUIRE) == 0) return ServeSlotState::running;
+    return __atomic_load_n(status, __ATOMIC_RELAXED) != 0 ? ServeSlotState::timed_out : ServeSlotState::finished;
 }
 
 }  // namespace proxmf

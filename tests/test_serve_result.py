@@ -23,3 +23,15 @@ def run(tmp_path, *flags, args=()):
 def test_timed_out_slot_is_never_finished(tmp_path):
     r = run(tmp_path)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_no_data_race(tmp_path):
+    """Under ThreadSanitizer: what follows done is read behind an acquire."""
+    probe = tmp_path / "probe.cpp"
+    probe.write_text("int main() { return 0; }")
+    exe = tmp_path / "probe"
+    b = subprocess.run(["g++", "-fsanitize=thread", str(probe), "-o", str(exe)], capture_output=True, text=True)
+    if b.returncode != 0 or subprocess.run([str(exe)]).returncode != 0:
+        pytest.skip("no ThreadSanitizer runtime here")
+    r = run(tmp_path, "-g", "-fsanitize=thread", args=("short",))
+    assert r.returncode == 0 and "WARNING: ThreadSanitizer" not in r.stderr, r.stdout + r.stderr
