@@ -15,6 +15,7 @@
 #include "../../include/proxmf.h"
 #include "nvtx_range.h"
 #include "internal.h"
+#include "sparse_rules.h"
 
 using namespace proxmf;
 
@@ -344,7 +345,7 @@ cudaError_t launch_step(crf_t h, const float *eta, int t, int update, double rel
         a.rel_tol = rel_tol;
         a.sym = h->mu_sym;
         if (pending) {
-            a.defer = sparse_blocks(h->N, h->L, h->sp_split);
+            a.defer = sparse_blocks(h->N, sparse_lanes(h->LP), h->sp_split);
             a.prev_pending = *pending;
             *pending = a.defer;
         }
@@ -601,9 +602,11 @@ crf_status crf_create(const crf_desc *desc, crf_t *out) {
     h->conn = d.topology == CRF_GRID8 ? 8 : 4;
     h->nd = h->conn == 8 ? 4 : 2;
     h->st = (cudaStream_t)d.stream;
-    int nbx, nby;
-    grid_tiles(h->H, h->W, &nbx, &nby);
-    h->nblk = nbx * nby;
+    if (!sparse) {
+        int nbx, nby;
+        grid_tiles(h->H, h->W, &nbx, &nby);
+        h->nblk = nbx * nby;
+    }
     h->dense = dense;
     h->N = h->H * h->W;
     if (dense) {
@@ -886,6 +889,7 @@ crf_status crf_set_graph(crf_t h, const float *mu, int64_t n_edges, const int32_
     for (int i = 0; i < h->L; ++i)
         for (int j = i + 1; j < h->L; ++j)
             if (m[(size_t)i * h->L + j] != m[(size_t)j * h->L + i]) sym = false;
+    if (!sparse_entries_fit(n_edges, sym)) return CRF_E_UNSUPPORTED;
     drop_graphs(h);   // they hold the old adjacency arrays and their split
     std::vector<int> optr, ocol, iptr, icol;
     std::vector<float> ow, iw;
@@ -933,7 +937,7 @@ crf_status crf_set_graph(crf_t h, const float *mu, int64_t n_edges, const int32_
     h->launches += sym ? 2 : 2;
     h->mu = m;
     h->mu_sym = sym;
-    h->sp_split = sparse_split(h->N, h->L, (int64_t)std::max(ocol.size(), icol.size()));
+    h->sp_split = sparse_split(h->N, sparse_lanes(h->LP), (int64_t)std::max(ocol.size(), icol.size()));
     h->lambda_valid = true;
     h->has_pairwise = true;
     h->fcur_valid = false;

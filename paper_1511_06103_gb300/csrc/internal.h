@@ -312,9 +312,6 @@ struct SparseStepLaunch {
     int defer, prev_pending; // deferred free energy in a loop, as for the dense steps
     bool sym;
 };
-int sparse_split(int N, int L, int64_t entries);   // entries: of the longer of the two adjacency arrays
-int sparse_blocks(int N, int L, int split);        // blocks, and free-energy partials, per instance
-int sparse_max_blocks(int N);
 cudaError_t launch_sparse_step(const SparseStepLaunch &a, cudaStream_t st);
 cudaError_t launch_sparse_degree(const int *ptr, const float *w, int N, unsigned *out_bits, cudaStream_t st);
 

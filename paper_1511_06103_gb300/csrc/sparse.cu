@@ -35,24 +35,23 @@
 #include "f32x2.cuh"
 #include "f_deferred.cuh"
 #include "internal.h"
+#include "sparse_rules.h"
 
 namespace proxmf {
 
 namespace {
 
-constexpr int kSW = 8;               // warps per block
+constexpr int kSW = kSparseWarps;
 constexpr int kST = kSW * 32;
-constexpr int kSparseBlocks = 4 * 152;
 
 // Lanes per variable and labels per lane.
 template <int LP>
 struct SparseGeom {
     static constexpr int V = LP == 2 ? 2 : 4;
-    static constexpr int GL = LP / V;                                          // lanes with labels
-    static constexpr int G = GL <= 1 ? 1 : GL <= 2 ? 2 : GL <= 4 ? 4 : 8;      // lanes used
-    static constexpr int ROW = G * V;                                          // padded label count
+    static constexpr int GL = LP / V;                   // lanes with labels
+    static constexpr int G = sparse_lanes(LP);          // lanes used
+    static constexpr int ROW = G * V;                   // padded label count
 };
-inline int sparse_lanes(int LP) { return LP <= 4 ? 1 : LP <= 8 ? 2 : LP <= 16 ? 4 : 8; }
 
 template <int V>
 __device__ __forceinline__ void vload(float (&v)[V], const float *p) {
@@ -84,8 +83,10 @@ __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, in
     constexpr int V = Gm::V;
 #pragma unroll
     for (int l = 0; l < V; ++l) S[l] = 0.f;
-    int e = e0 + part;
-    for (; e + 3 * split < e1; e += 4 * split) {
+    // unsigned: positions in the arrays may be near 2^31
+    const unsigned end = e1;
+    unsigned e = (unsigned)e0 + part;
+    for (; (int)(end - e) > 3 * split; e += 4 * split) {
         int c[4];
         float w[4], v[4][V];
 #pragma unroll
@@ -102,13 +103,13 @@ __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, in
                 for (int l = 0; l < V; ++l) S[l] = fmaf(w[j], v[j][l], S[l]);
         }
     }
-    if (e < e1) {
+    if ((int)(end - e) > 0) {
         // up to three more entries, together
         float w[3], v[3][V];
         int c[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const bool in = e + j * split < e1;
+            const bool in = (int)(end - e) > j * split;
             c[j] = in ? __ldg(col + e + j * split) : -1;
             w[j] = in ? __ldg(wt + e + j * split) : 0.f;
         }
@@ -139,12 +140,14 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
     __shared__ __align__(16) float sS[kSW][(SYM ? 1 : 2) * 32 * V];   // the S (and T) of a warp's lanes
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int N = a.N, L = a.L, split = a.split;
+    const int L = a.L, split = a.split;
+    const unsigned N = a.N;
     const size_t base = (size_t)b * N * LP;
     const int g = lane & (G - 1), part = (lane / G) & (split - 1);
     const int vpw = 32 / (G * split), slot = lane / (G * split);
     const bool has = g < Gm::GL;
-    const int first = (blockIdx.x * kSW + warp) * vpw, stride = gridDim.x * kSW * vpw;
+    const SparseWalk walk = sparse_walk(blockIdx.x, gridDim.x, warp, vpw);
+    const unsigned first = walk.first, stride = walk.stride;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the graph and mu do not change between steps
@@ -155,7 +158,7 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
         if (!SYM) mus[LP * ROW + e] = in ? a.mu[k * L + l] : 0.f;
     }
     int o0 = 0, o1 = 0, i0 = 0, i1 = 0;
-    auto bounds = [&](int i) {
+    auto bounds = [&](unsigned i) {
         if (i >= N) {
             o0 = o1 = i0 = i1 = 0;
             return;
@@ -182,8 +185,8 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
     }
     if (stopped) {
         // stopping rule met: carry the state through unchanged
-        for (int v0 = first; v0 < N; v0 += stride) {
-            const int i = v0 + slot;
+        for (unsigned v0 = first; v0 < N; v0 += stride) {
+            const unsigned i = v0 + slot;
             if (a.update && i < N && has && part == 0) {
                 const size_t o = base + (size_t)i * LP + g * V;
                 float v[V];
@@ -199,8 +202,8 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
     const float eta = a.eta[b];
     const float *qb = a.q_in + base + g * V;
     float fh = 0.f, fl = 0.f;   // compensated sum of this lane's F terms
-    for (int v0 = first; v0 < N; v0 += stride) {
-        const int i = v0 + slot;
+    for (unsigned v0 = first; v0 < N; v0 += stride) {
+        const unsigned i = v0 + slot;
         const bool act = i < N;
         const size_t o = base + (size_t)(act ? i : 0) * LP + (has ? g * V : 0);
         float s[V], u[V];
@@ -287,7 +290,7 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
 // step bound); scratch word as float bits (non-negative floats order as uints)
 __global__ void sparse_degree_kernel(const int *ptr, const float *w, int N, unsigned *out_bits) {
     float best = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)N; i += gridDim.x * blockDim.x) {
         float d = 0.f;
         for (int e = ptr[i]; e < ptr[i + 1]; ++e) d += fabsf(w[e]);
         best = fmaxf(best, d);
@@ -299,7 +302,7 @@ __global__ void sparse_degree_kernel(const int *ptr, const float *w, int N, unsi
 template <int LP>
 cudaError_t launch_lp(const SparseStepLaunch &a, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(sparse_blocks(a.N, a.L, a.split), a.B, 1);
+    cfg.gridDim = dim3(sparse_blocks(a.N, sparse_lanes(a.LP), a.split), a.B, 1);
     cfg.blockDim = dim3(kST, 1, 1);
     cfg.stream = st;
     // programmatic dependent launch: mu and the first list bounds are read
@@ -315,26 +318,8 @@ cudaError_t launch_lp(const SparseStepLaunch &a, cudaStream_t st) {
 
 }  // namespace
 
-// Lane groups per adjacency list: as many as it takes to have about 98304
-// threads (20 warps per SM), but no more than half the mean list length, so
-// that a group has at least two entries of its own on average.
-int sparse_split(int N, int L, int64_t entries) {
-    const int lanes = sparse_lanes(storage_labels(L));
-    int split = 1;
-    while (2 * split * lanes <= 32 && (int64_t)N * lanes * split < 98304 && entries >= (int64_t)4 * split * N)
-        split *= 2;
-    return split;
-}
-
-int sparse_blocks(int N, int L, int split) {
-    const int per = kSW * 32 / (sparse_lanes(storage_labels(L)) * split);
-    return std::min((N + per - 1) / per, kSparseBlocks);
-}
-
-int sparse_max_blocks(int N) { return std::min((N + kSW - 1) / kSW, kSparseBlocks); }
-
 cudaError_t launch_sparse_step(const SparseStepLaunch &a, cudaStream_t st) {
-    if (a.defer && a.defer != sparse_blocks(a.N, a.L, a.split)) return cudaErrorInvalidValue;
+    if (a.defer && a.defer != sparse_blocks(a.N, sparse_lanes(a.LP), a.split)) return cudaErrorInvalidValue;
     switch (a.LP) {
     case 2: return launch_lp<2>(a, st);
     case 4: return launch_lp<4>(a, st);
@@ -352,7 +337,7 @@ cudaError_t launch_sparse_step(const SparseStepLaunch &a, cudaStream_t st) {
 cudaError_t launch_sparse_degree(const int *ptr, const float *w, int N, unsigned *out_bits, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(out_bits, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
-    sparse_degree_kernel<<<std::min((N + 255) / 256, 1024), 256, 0, st>>>(ptr, w, N, out_bits);
+    sparse_degree_kernel<<<std::min((N - 1) / 256 + 1, 1024), 256, 0, st>>>(ptr, w, N, out_bits);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,57 @@
+// sparse_rules.h -- how the edge-list step (sparse.cu) deals variables and
+// adjacency lists out to lanes, warps and blocks.  Plain C++ (no CUDA headers), so
+// that the arithmetic is checked on the CPU at sizes no test allocates:
+// crf_create takes up to 2^31 - 1 variables, so index arithmetic past N is
+// unsigned (a stride is below 2^18) and sums that may pass 2^31 are 64-bit.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define PROXMF_HD __host__ __device__
+#else
+#define PROXMF_HD
+#endif
+
+namespace proxmf {
+
+constexpr int kSparseWarps = 8;                // warps per block
+constexpr int kSparseBlocks = 4 * 152;         // blocks per instance at most
+
+// Lanes that hold the labels of one variable (LP stored labels, a vector each).
+PROXMF_HD constexpr int sparse_lanes(int LP) { return LP <= 4 ? 1 : LP <= 8 ? 2 : LP <= 16 ? 4 : 8; }
+
+// Lane groups per adjacency list: as many as it takes to have about 98304
+// threads (20 warps per SM), but no more than half the mean list length, so
+// that a group has at least two entries of its own on average.  `entries` are
+// those of the longer of the two adjacency arrays.
+inline int sparse_split(int N, int lanes, int64_t entries) {
+    int split = 1;
+    while (2 * split * lanes <= 32 && (int64_t)N * lanes * split < 98304 && entries >= (int64_t)4 * split * N)
+        split *= 2;
+    return split;
+}
+
+// Blocks, and free-energy partials, per instance.
+inline int sparse_blocks(int N, int lanes, int split) {
+    const int64_t per = kSparseWarps * 32 / (lanes * split);
+    return (int)std::min<int64_t>((N + per - 1) / per, kSparseBlocks);
+}
+inline int sparse_max_blocks(int N) {
+    return (int)std::min<int64_t>(((int64_t)N + kSparseWarps - 1) / kSparseWarps, kSparseBlocks);
+}
+
+// The items a warp takes: first, first + stride, ... below n, `per` at a time.
+struct SparseWalk {
+    uint32_t first, stride;
+};
+PROXMF_HD inline SparseWalk sparse_walk(uint32_t block, uint32_t blocks, uint32_t warp, uint32_t per) {
+    return {(block * kSparseWarps + warp) * per, blocks * kSparseWarps * per};
+}
+
+// The adjacency arrays are indexed by int: n_edges edges make as many entries, or
+// twice as many when a list holds both directions (symmetric mu).
+inline bool sparse_entries_fit(int64_t n_edges, bool both) { return n_edges * (both ? 2 : 1) <= INT32_MAX; }
+
+}  // namespace proxmf
