@@ -39,6 +39,8 @@ struct crf_s {
     float *sp_out_w = nullptr, *sp_in_w = nullptr;
     double *sp_nu = nullptr;     // [2] extreme eigenvalues of C mu C
     int sp_split = 1;            // lane groups per adjacency list (sparse_split)
+    int *sp_long = nullptr;      // variables with a long list (SparseStepLaunch::long_ids)
+    int sp_n_block_long = 0, sp_n_long = 0, sp_long_list = 0;
     // fully connected model
     bool dense = false;
     int N = 0;                   // variables per instance
@@ -182,7 +184,7 @@ void free_all(crf_t h) {
     if (h->status) cudaFree(h->status);
     if (h->mu_pairs) cudaFree(h->mu_pairs);
     if (h->mu_tc) cudaFree(h->mu_tc);
-    int *ip[] = {h->sp_out_ptr, h->sp_out_col, h->sp_in_ptr, h->sp_in_col};
+    int *ip[] = {h->sp_out_ptr, h->sp_out_col, h->sp_in_ptr, h->sp_in_col, h->sp_long};
     for (int *p : ip)
         if (p) cudaFree(p);
     if (h->sp_out_w) cudaFree(h->sp_out_w);
@@ -339,6 +341,10 @@ cudaError_t launch_step(crf_t h, const float *eta, int t, int update, double rel
         a.LP = h->LP;
         a.fpitch = f_pitch(h);
         a.split = h->sp_split;
+        a.long_ids = h->sp_long;
+        a.n_block_long = h->sp_n_block_long;
+        a.n_long = h->sp_n_long;
+        a.long_list = h->sp_long_list;
         a.t = t;
         a.trace_cap = h->trace_cap;
         a.update = update;
@@ -900,6 +906,28 @@ crf_status crf_set_graph(crf_t h, const float *mu, int64_t n_edges, const int32_
     CK(h, upload(&h->sp_in_ptr, iptr, h->st));
     CK(h, upload(&h->sp_in_col, icol, h->st));
     CK(h, upload(&h->sp_in_w, iw, h->st));
+    const int lanes = sparse_lanes(h->LP);
+    const int64_t entries = (int64_t)std::max(ocol.size(), icol.size());
+    h->sp_split = sparse_split(h->N, lanes, entries);
+    auto list_of = [&](int i) {
+        return std::max(optr[(size_t)i + 1] - optr[i], iptr[(size_t)i + 1] - iptr[i]);
+    };
+    int longest = 0;
+    for (int i = 0; i < h->N; ++i) longest = std::max(longest, list_of(i));
+    h->sp_long_list = sparse_long_list(h->N, lanes, h->sp_split, entries, longest);
+    const int block_list = std::max(h->sp_long_list, sparse_block_list(lanes));
+    std::vector<int> longs, warp_longs;
+    for (int i = 0; i < h->N && longest > h->sp_long_list; ++i) {
+        const int n = list_of(i);
+        if (n > block_list)
+            longs.push_back(i);
+        else if (n > h->sp_long_list)
+            warp_longs.push_back(i);
+    }
+    h->sp_n_block_long = (int)longs.size();
+    h->sp_n_long = (int)warp_longs.size();
+    longs.insert(longs.end(), warp_longs.begin(), warp_longs.end());
+    CK(h, upload(&h->sp_long, longs, h->st));
     CK(h, cudaMemcpyAsync(h->mu_dev, m.data(), LL * sizeof(float), cudaMemcpyHostToDevice, h->st));
     // step bound (see proxmf.h): the largest summed |w| per variable, and
     // the spectrum of C mu C (symmetric mu) or ||mu||_F
@@ -937,7 +965,6 @@ crf_status crf_set_graph(crf_t h, const float *mu, int64_t n_edges, const int32_
     h->launches += sym ? 2 : 2;
     h->mu = m;
     h->mu_sym = sym;
-    h->sp_split = sparse_split(h->N, sparse_lanes(h->LP), (int64_t)std::max(ocol.size(), icol.size()));
     h->lambda_valid = true;
     h->has_pairwise = true;
     h->fcur_valid = false;

@@ -306,7 +306,11 @@ struct SparseStepLaunch {
     double *f_trace, *f_cur;
     int *done, *status;
     int B, N, L, LP;
-    int split;               // lanes that share an adjacency list (sparse_split)
+    int split;               // lane groups that share an adjacency list (sparse_split)
+    // variables with a list longer than long_list (sparse_long_list): first those
+    // whose list a block walks (sparse_block_list), then those of a warp
+    const int *long_ids;
+    int n_block_long, n_long, long_list;
     int t, trace_cap, update;
     double rel_tol;
     int defer, prev_pending; // deferred free energy in a loop, as for the dense steps

@@ -26,6 +26,7 @@
 // warp per list, four variables in turn and the blocks' ticket.  Twice, four
 // and fourteen times as many blocks: 72, 78 and 104 us on the random graph; five
 // or six resident blocks of fewer registers: 80 and 83 us.
+// Lists far longer than the mean have passes of their own (LONG, sparse_rules.h).
 // Blocks walk the variables grid-stride, at most kSparseBlocks of them (four
 // per SM, all resident), so that the next step can sum their free-energy partials
 // (f_deferred.cuh) while its lists are in flight.
@@ -72,13 +73,14 @@ __device__ __forceinline__ void vstore(float *p, const float (&v)[V]) {
         *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
 }
 
-// The lane's labels of sum_e w_e q[col_e] over entries e0 + part, + split, ...
-// of one adjacency list, summed over the variable's lane groups.  q points at
-// the lane's labels of variable 0; lanes past the labels (has = false) add 0.
+// The lane's labels of sum_e w_e q[col_e] over entries e0 + part, + step, ... of
+// one adjacency list, summed over the `groups` lane groups of the warp that share
+// it (step = groups unless warps share it too).  q points at the lane's labels of
+// variable 0; lanes past the labels (has = false) add 0.
 template <int LP>
 __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, int e1, const int *__restrict__ col,
-                                       const float *__restrict__ wt, const float *__restrict__ q, int part, int split,
-                                       bool has) {
+                                       const float *__restrict__ wt, const float *__restrict__ q, int part, int step,
+                                       int groups, bool has) {
     using Gm = SparseGeom<LP>;
     constexpr int V = Gm::V;
 #pragma unroll
@@ -86,13 +88,13 @@ __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, in
     // unsigned: positions in the arrays may be near 2^31
     const unsigned end = e1;
     unsigned e = (unsigned)e0 + part;
-    for (; (int)(end - e) > 3 * split; e += 4 * split) {
+    for (; (int)(end - e) > 3 * step; e += 4 * step) {
         int c[4];
         float w[4], v[4][V];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            c[j] = __ldg(col + e + j * split);
-            w[j] = __ldg(wt + e + j * split);
+            c[j] = __ldg(col + e + j * step);
+            w[j] = __ldg(wt + e + j * step);
         }
         if (has) {
 #pragma unroll
@@ -109,9 +111,9 @@ __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, in
         int c[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const bool in = (int)(end - e) > j * split;
-            c[j] = in ? __ldg(col + e + j * split) : -1;
-            w[j] = in ? __ldg(wt + e + j * split) : 0.f;
+            const bool in = (int)(end - e) > j * step;
+            c[j] = in ? __ldg(col + e + j * step) : -1;
+            w[j] = in ? __ldg(wt + e + j * step) : 0.f;
         }
 #pragma unroll
         for (int j = 0; j < 3; ++j)
@@ -124,13 +126,17 @@ __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, in
             }
     }
     __syncwarp();
-    for (int o = split / 2 * Gm::G; o >= Gm::G; o >>= 1) {
+    for (int o = groups / 2 * Gm::G; o >= Gm::G; o >>= 1) {
 #pragma unroll
         for (int l = 0; l < V; ++l) S[l] += __shfl_xor_sync(0xffffffffu, S[l], o);
     }
 }
 
-template <int LP, bool SYM>
+// LONG: the graph has lists far longer than its mean (sparse_long_list).  A warp
+// takes as long as its longest list, so those are walked first, by a whole block
+// or a whole warp each, and passed over when the lane groups take theirs.  A form
+// of its own, since the passes cost the other graphs 5 to 8 %.
+template <int LP, bool SYM, bool LONG>
 __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __grid_constant__ SparseStepLaunch a) {
     using Gm = SparseGeom<LP>;
     constexpr int V = Gm::V, G = Gm::G, ROW = Gm::ROW;
@@ -140,14 +146,33 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
     __shared__ __align__(16) float sS[kSW][(SYM ? 1 : 2) * 32 * V];   // the S (and T) of a warp's lanes
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int L = a.L, split = a.split;
+    __shared__ __align__(16) float sB[LONG ? (SYM ? 1 : 2) * kSW * ROW : 4];   // the warps' shares of a list
+    const int L = a.L;
     const unsigned N = a.N;
     const size_t base = (size_t)b * N * LP;
-    const int g = lane & (G - 1), part = (lane / G) & (split - 1);
-    const int vpw = 32 / (G * split), slot = lane / (G * split);
+    const int g = lane & (G - 1);
     const bool has = g < Gm::GL;
-    const SparseWalk walk = sparse_walk(blockIdx.x, gridDim.x, warp, vpw);
-    const unsigned first = walk.first, stride = walk.stride;
+    // who walks a list: 2 a block, 1 a warp, 0 `split` lane groups; and the pass's
+    // items, of which this lane works on first + slot, + stride, ...
+    int mode = LONG ? 2 : 0;
+    int split, part, slot;
+    unsigned items, first, stride;
+    auto deal = [&] {
+        split = mode ? 32 / G : a.split;
+        const int per = 32 / (G * split);   // items of a warp at a time
+        part = (lane / G) & (split - 1);
+        slot = lane / (G * split);
+        const SparseWalk walk = sparse_walk(blockIdx.x, gridDim.x, warp, per);
+        first = walk.first;
+        stride = walk.stride;
+        items = mode == 0 ? N : (unsigned)(mode == 1 ? a.n_long : a.n_block_long);
+        if (mode == 2) {
+            part += warp * split;
+            first = blockIdx.x;
+            stride = gridDim.x;
+        }
+    };
+    deal();
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the graph and mu do not change between steps
@@ -158,8 +183,14 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
         if (!SYM) mus[LP * ROW + e] = in ? a.mu[k * L + l] : 0.f;
     }
     int o0 = 0, o1 = 0, i0 = 0, i1 = 0;
+    unsigned next = N;   // LONG: the variable of the item whose lists were read last (N: none)
     auto bounds = [&](unsigned i) {
-        if (i >= N) {
+        if constexpr (LONG) {
+            o0 = o1 = i0 = i1 = 0;
+            next = N;
+            if (i >= items) return;
+            if (mode) i = (unsigned)__ldg(a.long_ids + (mode == 1 ? a.n_block_long : 0) + i);
+        } else if (i >= N) {
             o0 = o1 = i0 = i1 = 0;
             return;
         }
@@ -168,6 +199,12 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
         if (!SYM) {
             i0 = __ldg(a.in_ptr + i);
             i1 = __ldg(a.in_ptr + i + 1);
+        }
+        if constexpr (LONG) {
+            if (mode == 0 && (o1 - o0 > a.long_list || i1 - i0 > a.long_list))
+                o0 = o1 = i0 = i1 = 0;   // walked before
+            else
+                next = i;
         }
     };
     bounds(first + slot);
@@ -185,6 +222,10 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
     }
     if (stopped) {
         // stopping rule met: carry the state through unchanged
+        if constexpr (LONG) {
+            mode = 0;
+            deal();
+        }
         for (unsigned v0 = first; v0 < N; v0 += stride) {
             const unsigned i = v0 + slot;
             if (a.update && i < N && has && part == 0) {
@@ -202,8 +243,17 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
     const float eta = a.eta[b];
     const float *qb = a.q_in + base + g * V;
     float fh = 0.f, fl = 0.f;   // compensated sum of this lane's F terms
-    for (unsigned v0 = first; v0 < N; v0 += stride) {
-        const unsigned i = v0 + slot;
+    for (unsigned v0 = first;; v0 += stride) {
+        if constexpr (LONG) {
+            while (v0 >= items && mode > 0) {   // next pass
+                --mode;
+                deal();
+                v0 = first;
+                bounds(v0 + slot);
+            }
+        }
+        if (v0 >= items) break;
+        const unsigned i = LONG ? next : v0 + slot;
         const bool act = i < N;
         const size_t o = base + (size_t)(act ? i : 0) * LP + (has ? g * V : 0);
         float s[V], u[V];
@@ -211,9 +261,29 @@ __global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __g
         vload<V>(u, a.U + o);
         // a1: neighbour sums
         float S[V], T[V];
-        gather<LP>(S, o0, o1, a.out_col, a.out_w, qb, part, split, has);
-        if (!SYM) gather<LP>(T, i0, i1, a.in_col, a.in_w, qb, part, split, has);
-        bounds(i + stride);   // of the next variable
+        const int step = LONG && mode == 2 ? kSW * split : split;
+        gather<LP>(S, o0, o1, a.out_col, a.out_w, qb, part, step, split, has);
+        if (!SYM) gather<LP>(T, i0, i1, a.in_col, a.in_w, qb, part, step, split, has);
+        if constexpr (LONG) {
+            if (mode == 2) {   // the whole block has this variable: its warps' shares, in warp order
+                if (lane < G) {
+                    vstore<V>(sB + warp * ROW + g * V, S);
+                    if (!SYM) vstore<V>(sB + (kSW + warp) * ROW + g * V, T);
+                }
+                __syncthreads();
+#pragma unroll
+                for (int l = 0; l < V; ++l) {
+                    S[l] = T[l] = 0.f;
+#pragma unroll
+                    for (int w = 0; w < kSW; ++w) {
+                        S[l] += sB[w * ROW + g * V + l];
+                        if (!SYM) T[l] += sB[(kSW + w) * ROW + g * V + l];
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        bounds(v0 + slot + stride);   // of the next variable
         // m_l = sum_k mu[l][k] S_k (+ sum_k mu[k][l] T_k), S through the warp's rows
         vstore<V>(&sS[warp][lane * V], S);
         if (!SYM) vstore<V>(&sS[warp][32 * V + lane * V], T);
@@ -312,8 +382,11 @@ cudaError_t launch_lp(const SparseStepLaunch &a, cudaStream_t st) {
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
-    return a.sym ? cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, true>, a)
-                 : cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, false>, a);
+    if (a.n_block_long + a.n_long > 0)
+        return a.sym ? cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, true, true>, a)
+                     : cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, false, true>, a);
+    return a.sym ? cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, true, false>, a)
+                 : cudaLaunchKernelEx(&cfg, sparse_step_kernel<LP, false, false>, a);
 }
 
 }  // namespace

@@ -19,6 +19,9 @@ int main() {
             for (long long deg : {0LL, 1LL, 40LL, 3000LL}) {
                 const int split = sparse_split(N, lanes, deg * N), per = 32 / (lanes * split);
                 const int blocks = sparse_blocks(N, lanes, split);
+                const int block = sparse_block_list(lanes), longest = N / 2;
+                const int lng = sparse_long_list(N, lanes, split, deg * N, longest);
+                check(lng == INT32_MAX || (lng >= 4 * deg && lng >= 32 && longest > lng) || lng == block, "long list", N, lng);
                 check(split >= 1 && per >= 1, "split", N, split);
                 check(blocks >= 1 && blocks <= sparse_max_blocks(N) && blocks <= kSparseBlocks, "blocks", N, blocks);
                 check((long long)blocks * kSparseWarps * per >= N || blocks == kSparseBlocks, "blocks cover N", N, blocks);
