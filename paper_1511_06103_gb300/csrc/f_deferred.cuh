@@ -50,28 +50,27 @@ __device__ __forceinline__ bool f_deferred(const Args &a, int b, int t_prev, int
     return stop;
 }
 
-// A block's share of F (thread 0 holds it): deferred to the next step, or
-// summed by the last of the instance's n blocks behind a ticket, whose threads
-// take fixed strided subsets of the partials and then a fixed-shape tree, so
+// Where partial `part` of this launch goes: slot t & 1 when deferred, else slot 0.
+template <class Args>
+__device__ __forceinline__ double *f_partial(const Args &a, int b, int part) {
+    return a.partial + ((size_t)(a.defer ? a.t & 1 : 0) * a.B + b) * a.fpitch + part;
+}
+
+// Not deferred: the n partials that the instance's `blocks` blocks have stored
+// (thread 0's, or before a block barrier) are summed by the last of them behind a
+// ticket, whose threads take fixed strided subsets and then a fixed-shape tree, so
 // F does not depend on which block is last.
 template <int NT, class Args>
-__device__ __forceinline__ void f_finish(const Args &a, int b, int part, int n, double bs, double *red,
-                                               int &is_last) {
+__device__ __forceinline__ void f_ticket(const Args &a, int b, int blocks, int n, double *red, int &is_last) {
     const int tid = threadIdx.x;
-    const size_t P = a.fpitch;
-    if (a.defer) {
-        if (tid == 0) a.partial[((size_t)(a.t & 1) * a.B + b) * P + part] = bs;
-        return;
-    }
     if (tid == 0) {
-        a.partial[(size_t)b * P + part] = bs;
         __threadfence();
-        is_last = atomicAdd(a.counter + b, 1u) == (unsigned)(n - 1);
+        is_last = atomicAdd(a.counter + b, 1u) == (unsigned)(blocks - 1);
     }
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    const double F = f_sum_partials<NT>(a.partial + (size_t)b * P, n, red);
+    const double F = f_sum_partials<NT>(a.partial + (size_t)b * a.fpitch, n, red);
     if (tid != 0) return;
     a.f_cur[b] = F;
     if (!isfinite(F)) atomicExch(a.status, -6);
@@ -83,6 +82,15 @@ __device__ __forceinline__ void f_finish(const Args &a, int b, int part, int n, 
         }
     }
     a.counter[b] = 0u;
+}
+
+// A block's share of F (thread 0 holds it), one of n: deferred to the next step,
+// or summed by the last of the instance's n blocks.
+template <int NT, class Args>
+__device__ __forceinline__ void f_finish(const Args &a, int b, int part, int n, double bs, double *red,
+                                         int &is_last) {
+    if (threadIdx.x == 0) *f_partial(a, b, part) = bs;
+    if (!a.defer) f_ticket<NT>(a, b, n, n, red, is_last);
 }
 
 }  // namespace proxmf
