@@ -351,7 +351,7 @@ cudaError_t launch_step(crf_t h, const float *eta, int t, int update, double rel
         a.rel_tol = rel_tol;
         a.sym = h->mu_sym;
         if (pending) {
-            a.defer = sparse_blocks(h->N, sparse_lanes(h->LP), h->sp_split);
+            a.defer = sparse_blocks(h->N, sparse_lanes(h->LP), h->sp_split, h->mu_sym);
             a.prev_pending = *pending;
             *pending = a.defer;
         }

@@ -27,9 +27,10 @@
 // and fourteen times as many blocks: 72, 78 and 104 us on the random graph; five
 // or six resident blocks of fewer registers: 80 and 83 us.
 // Lists far longer than the mean have passes of their own (LONG, sparse_rules.h).
-// Blocks walk the variables grid-stride, at most kSparseBlocks of them (four
-// per SM, all resident), so that the next step can sum their free-energy partials
-// (f_deferred.cuh) while its lists are in flight.
+// Blocks walk the variables grid-stride, at most as many as run at a time (four per
+// SM, three for asymmetric mu, whose second product takes 80 registers), so that all
+// have the same share of the time and the next step has few free-energy partials to
+// sum (f_deferred.cuh).
 #include <cmath>
 
 #include "dfloat.cuh"
@@ -137,7 +138,7 @@ __device__ __forceinline__ void gather(float (&S)[SparseGeom<LP>::V], int e0, in
 // or a whole warp each, and passed over when the lane groups take theirs.  A form
 // of its own, since the passes cost the other graphs 5 to 8 %.
 template <int LP, bool SYM, bool LONG>
-__global__ void __launch_bounds__(kST, SYM ? 4 : 3) sparse_step_kernel(const __grid_constant__ SparseStepLaunch a) {
+__global__ void __launch_bounds__(kST, sparse_per_sm(SYM)) sparse_step_kernel(const __grid_constant__ SparseStepLaunch a) {
     using Gm = SparseGeom<LP>;
     constexpr int V = Gm::V, G = Gm::G, ROW = Gm::ROW;
     __shared__ double red[kSW];
@@ -372,7 +373,7 @@ __global__ void sparse_degree_kernel(const int *ptr, const float *w, int N, unsi
 template <int LP>
 cudaError_t launch_lp(const SparseStepLaunch &a, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(sparse_blocks(a.N, sparse_lanes(a.LP), a.split), a.B, 1);
+    cfg.gridDim = dim3(sparse_blocks(a.N, sparse_lanes(a.LP), a.split, a.sym), a.B, 1);
     cfg.blockDim = dim3(kST, 1, 1);
     cfg.stream = st;
     // programmatic dependent launch: mu and the first list bounds are read
@@ -392,7 +393,7 @@ cudaError_t launch_lp(const SparseStepLaunch &a, cudaStream_t st) {
 }  // namespace
 
 cudaError_t launch_sparse_step(const SparseStepLaunch &a, cudaStream_t st) {
-    if (a.defer && a.defer != sparse_blocks(a.N, sparse_lanes(a.LP), a.split)) return cudaErrorInvalidValue;
+    if (a.defer && a.defer != sparse_blocks(a.N, sparse_lanes(a.LP), a.split, a.sym)) return cudaErrorInvalidValue;
     switch (a.LP) {
     case 2: return launch_lp<2>(a, st);
     case 4: return launch_lp<4>(a, st);

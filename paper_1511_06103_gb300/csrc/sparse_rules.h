@@ -17,7 +17,13 @@
 namespace proxmf {
 
 constexpr int kSparseWarps = 8;                // warps per block
-constexpr int kSparseBlocks = 4 * 152;         // blocks per instance at most
+// Blocks per instance at most: those that run at a time on the 152 SMs, by the
+// kernel's registers.  (In a batch every instance has that many, so that its free
+// energy has the same bits as alone; they run in whole waves.)  With four an SM for
+// asymmetric mu too, a third of whose blocks then ran in a second wave, 20 steps on
+// N = 262144 with 8 entries a list took 3100 us at 21 labels, now 2230, and 612 at 8, now 515.
+PROXMF_HD constexpr int sparse_per_sm(bool sym) { return sym ? 4 : 3; }
+constexpr int sparse_resident(bool sym) { return 152 * sparse_per_sm(sym); }
 
 // Lanes that hold the labels of one variable (LP stored labels, a vector each).
 PROXMF_HD constexpr int sparse_lanes(int LP) { return LP <= 4 ? 1 : LP <= 8 ? 2 : LP <= 16 ? 4 : 8; }
@@ -53,12 +59,12 @@ inline int sparse_long_list(int N, int lanes, int split, int64_t entries, int lo
 }
 
 // Blocks, and free-energy partials, per instance.
-inline int sparse_blocks(int N, int lanes, int split) {
+inline int sparse_blocks(int N, int lanes, int split, bool sym) {
     const int64_t per = kSparseWarps * 32 / (lanes * split);
-    return (int)std::min<int64_t>((N + per - 1) / per, kSparseBlocks);
+    return (int)std::min<int64_t>((N + per - 1) / per, sparse_resident(sym));
 }
 inline int sparse_max_blocks(int N) {
-    return (int)std::min<int64_t>(((int64_t)N + kSparseWarps - 1) / kSparseWarps, kSparseBlocks);
+    return (int)std::min<int64_t>(((int64_t)N + kSparseWarps - 1) / kSparseWarps, sparse_resident(true));
 }
 
 // The items a warp takes: first, first + stride, ... below n, `per` at a time.
