@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kST, sparse_per_sm(SYM)) sparse_step_kernel(co
     const float eta = a.eta[b];
     const float *qb = a.q_in + base + g * V;
     float fh = 0.f, fl = 0.f;   // compensated sum of this lane's F terms
-    for (unsigned v0 = first;; v0 += stride) {
+    auto more = [&](unsigned &v0) {
         if constexpr (LONG) {
             while (v0 >= items && mode > 0) {   // next pass
                 --mode;
@@ -253,7 +253,9 @@ __global__ void __launch_bounds__(kST, sparse_per_sm(SYM)) sparse_step_kernel(co
                 bounds(v0 + slot);
             }
         }
-        if (v0 >= items) break;
+        return v0 < items;
+    };
+    for (unsigned v0 = first; more(v0); v0 += stride) {
         const unsigned i = LONG ? next : v0 + slot;
         const bool act = i < N;
         const size_t o = base + (size_t)(act ? i : 0) * LP + (has ? g * V : 0);
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(kST, sparse_per_sm(SYM)) sparse_step_kernel(co
                 __syncthreads();
             }
         }
-        bounds(v0 + slot + stride);   // of the next variable
+        bounds((LONG ? v0 + slot : i) + stride);   // of the next variable
         // m_l = sum_k mu[l][k] S_k (+ sum_k mu[k][l] T_k), S through the warp's rows
         vstore<V>(&sS[warp][lane * V], S);
         if (!SYM) vstore<V>(&sS[warp][32 * V + lane * V], T);
