@@ -149,17 +149,18 @@ struct DenseShares {
 
 // Warps of a share: as few as take no more chunks each than twelve would (fewer rounds
 // where a CTA has several shares); beyond one chunk each a multiple of four, so that the
-// SM's four schedulers have the same work.
+// SM's four schedulers have the same work: that is eight or twelve.
 inline int dense_share_warps(int nchunk, int shares) {
     const int most = (nchunk + shares - 1) / shares, turns = (most + kNW - 1) / kNW;
     return turns == 1 ? most : ((most + turns - 1) / turns + 3) / 4 * 4;
 }
 
-// SHARE: a CTA of the cluster for each share of k.  FEW, ONE: shares / nc of them on
+// SHARE, SHARE8: a CTA of the cluster for each share of k, its twelve or eight warps (a
+// constant: 0.5 % of a step at N = 9216).  FEW, ONE: shares / nc of them on
 // each of nc CTAs (ONE: nc = 1), in the same sums bit for bit: the (share, warp) pairs
 // are dealt to the twelve warps in rounds, and after each round the threads add its sums
 // on to the shares' (ONE: finished shares are added up as they come).
-enum DenseForm { SHARE, FEW, ONE };
+enum DenseForm { SHARE, SHARE8, FEW, ONE };
 
 template <int LP, DenseForm FORM>
 __global__ void __launch_bounds__(kDT, 1)
@@ -177,14 +178,14 @@ dense_step_f32_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int N = a.N, L = a.L, row0 = tile * kTM;
     uint8_t *base = dsm + ((128u - (tc::smem_u32(dsm) & 127u)) & 127u);
-    constexpr bool MULTI = FORM != SHARE;
+    constexpr bool MULTI = FORM == FEW || FORM == ONE;
     constexpr int RING = FORM == FEW ? G::FEW_RING : G::RING, DEPTH = FORM == FEW ? G::FEW_DEPTH : kDepth;
     uint8_t *ring = base + warp * RING;
     float *Sc = reinterpret_cast<float *>(base + (size_t)kNW * RING);   // [own shares][LP][kTM]: the CTA's sums
 
     // the warp's chunks of k: cw, cw + spw, ..., n of them
     const DenseShares sh{a.nchunk, MULTI ? a.shares : nc, a.share_warps};
-    const int own = MULTI ? a.shares / nc : 1, spw = a.share_warps;
+    const int own = MULTI ? a.shares / nc : 1, spw = MULTI ? a.share_warps : FORM == SHARE8 ? 8 : kNW;
     int cw, n;
     auto deal = [&](int round) {
         const int pair = round * kNW + warp, j = MULTI ? pair / spw : 0, w = pair - j * spw, share = rank * own + j;
@@ -397,7 +398,7 @@ dense_step_f32_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     for (int e = tid; e < LP * nr; e += kDT) {
         const int l = e / nr, r = e - l * nr;
         float t = 0.f;
-        if constexpr (FORM == SHARE) {
+        if constexpr (!MULTI) {
             for (int c = 0; c < nc; ++c) t += cluster.map_shared_rank(Sc, c)[l * kTM + r0 + r];
         } else if constexpr (FORM == ONE) {
             t = Sc[e];
@@ -464,13 +465,18 @@ dense_step_f32_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 // error.
 template <int LP>
 int f32_device() {
-    static SmemOptIn optin[3];
+    static std::atomic<unsigned long long> ready{0ull};   // a bit per device
+    static SmemOptIn optin[4];
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        smem_optin(optin[0], dense_step_f32_kernel<LP, SHARE>, DenseF32Geom<LP>::smem) != cudaSuccess ||
+    if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if ((ready.load(std::memory_order_acquire) & bit) != 0ull) return dev;
+    if (smem_optin(optin[0], dense_step_f32_kernel<LP, SHARE>, DenseF32Geom<LP>::smem) != cudaSuccess ||
+        smem_optin(optin[3], dense_step_f32_kernel<LP, SHARE8>, DenseF32Geom<LP>::smem) != cudaSuccess ||
         smem_optin(optin[1], dense_step_f32_kernel<LP, FEW>, DenseF32Geom<LP>::few_smem) != cudaSuccess ||
         smem_optin(optin[2], dense_step_f32_kernel<LP, ONE>, DenseF32Geom<LP>::one_smem) != cudaSuccess)
         return -1;
+    ready.fetch_or(bit, std::memory_order_acq_rel);
     return dev;
 }
 
@@ -596,7 +602,12 @@ template <int LP>
 cudaError_t launch_f32(cudaLaunchConfig_t &cfg, const CUtensorMap &tmK, const DenseF32Args &a, int nc) {
     using G = DenseF32Geom<LP>;
     cfg.dynamicSmemBytes = nc == a.shares ? G::smem : nc == 1 ? G::one_smem : G::few_smem;
-    if (nc == a.shares) return cudaLaunchKernelEx(&cfg, dense_step_f32_kernel<LP, SHARE>, tmK, a);
+    if (nc == a.shares) {
+        // one chunk a warp at most: any stride
+        const bool eight = a.share_warps == 8 && a.nchunk > 8 * a.shares;
+        return eight ? cudaLaunchKernelEx(&cfg, dense_step_f32_kernel<LP, SHARE8>, tmK, a)
+                     : cudaLaunchKernelEx(&cfg, dense_step_f32_kernel<LP, SHARE>, tmK, a);
+    }
     if (nc == 1) return cudaLaunchKernelEx(&cfg, dense_step_f32_kernel<LP, ONE>, tmK, a);
     return cudaLaunchKernelEx(&cfg, dense_step_f32_kernel<LP, FEW>, tmK, a);
 }
