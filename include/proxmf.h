@@ -345,7 +345,8 @@ crf_status mf_grid_step_noalloc(int32_t topology, int32_t n_labels, int64_t heig
  * `iters` proximal steps -- one graph launch per step, holding a persistent
  * kernel for each group of requests in flight.  A request stops after max_iters steps or when
  * |F^t - F^{t-1}| <= rel_tol |F^t| (Sec. 3.1), exactly as mf_iterate would
- * stop it, and its arithmetic does not depend on the other requests.
+ * stop it, and its arithmetic does not depend on the other requests (against a
+ * solve of its own its marginals differ by FP32 rounding).
  * eta <= 0 asks for eta = 1/(1 + D max|nu|) with D the largest weighted degree
  * and nu the eigenvalues of C mu C: an upper bound of the step-size constant
  * of Sec. 3.2 (so the descent guarantee holds) that costs no iteration; it

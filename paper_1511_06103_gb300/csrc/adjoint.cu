@@ -19,8 +19,8 @@
 // separate pass over the pixels); gm = -eta ga is applied as a factor at the
 // end of each product.  The dmu contribution of the tile is a small block
 // GEMM [ga | q]^T [S | Gout] over its 128 pixels, register-tiled 8 x 4.
-// What bounds it is the shared-memory pipe (75 % of its wavefronts over a
-// launch), so its accesses are laid out for that: rows spread over the banks,
+// What bounds it is the shared-memory pipe (64 % of its wavefronts over a launch,
+// at 12 warps an SM), so its accesses are laid out for that: rows spread over the banks,
 // own rows read as vectors, the block GEMM at six loads for 64 FMAs.  Two threads
 // a pixel (24 warps an SM instead of 12) read ga, q and the sums twice and took
 // 5.60 ms a training step (ten steps, 16 x 256 x 256, 21 labels) against 5.34 with

@@ -13,7 +13,8 @@
 //      requests, side by side, and the launch that ends the iteration
 //      (serve.cuh), once per requested iteration.
 // Requests therefore join and leave between iterations while the others keep
-// running, and every request's arithmetic is that of a solve on its own.
+// running, and a request's arithmetic does not depend on them (it agrees with a
+// handle's solve within rounding: the tiles form their sums in another order).
 //
 // No step waits for the device except to recycle host staging memory: the
 // uploads of an admission and the download of a result go through a ring of

@@ -47,7 +47,7 @@ struct ServeTable {
 
 // Groups of slots, each with its own kernel and tile table:
 //  0  two labels: little work a tile, so what counts is how many tiles an SM
-//     holds; its kernel is compiled for that path alone and takes 64 registers
+//     holds; its kernel is compiled for that path alone and takes 56 registers
 //     instead of the 128 that the longest label path needs;
 //  1  symmetric mu, 3..21 kernel labels: two pixels a thread on tiles that the
 //     TMA fetches one ahead (serve_pairs_kernel);
