@@ -59,6 +59,7 @@ struct crf_s {
     float *adapt_d = nullptr;    // [B] d of the adaptive binary step (or d0 of Adam)
     bool adapt_active = false;   // set while mf_iterate runs the adaptive rule
     float *mom = nullptr, *vv = nullptr;   // [B][N][LP] momentum / Adam state (allocated on first use)
+    bool plain_first = false;    // no kernel since crf_set_unary (GridStepLaunch::plain)
     int rule_kernel = 0;         // 1 momentum, 2 Adam, 3 ADHOC while mf_iterate runs them
     float gamma1 = 0.f, gamma2 = 0.f, eps = 0.f;
     float *eta_auto = nullptr;   // [B]
@@ -373,6 +374,7 @@ cudaError_t launch_step(crf_t h, const float *eta, int t, int update, double rel
     GridStepLaunch a = step_args(h, eta, t, update, rel_tol);
     if (!update || rel_tol <= 0) a.done = nullptr;
     a.tc = h->bf16 && update && !fp32;
+    a.plain = pending && t == 0 && h->plain_first;
     if (pending) {
         const int d = update ? grid_step_fparts(a) : 0;
         if (*pending && !d) {
@@ -1086,6 +1088,8 @@ crf_status mf_iterate(crf_t h, const mf_params *p, int32_t *iters_done) {
         }
         return cudaSuccess;
     };
+    // with a fixed step, or from q^0, a small kernel lies between the unaries and the loop
+    h->plain_first = eta == h->eta_auto && !p->reset;
     h->adapt_active = p->rule == MF_RULE_ADAPTIVE;
     h->rule_kernel = p->rule == MF_RULE_MOMENTUM ? 1 : (p->rule == MF_RULE_ADAM ? 2 : (p->rule == MF_RULE_ADHOC ? 3 : 0));
     h->gamma1 = (float)p->gamma1;

@@ -918,8 +918,8 @@ cudaError_t launch_grid_step_lt(const GridStepLaunch &l, cudaStream_t st) {
             GridTmaTcMaps maps;
             const cudaError_t e = encode_grid_tc_maps(&maps, l, TG::LP, TG::CS, TG::C16, TG::UP);
             if (e != cudaSuccess) return e;
-            return l.conn == 8 ? launch_grid_tma_tc<LT, 8>(maps, a, grid, st)
-                               : launch_grid_tma_tc<LT, 4>(maps, a, grid, st);
+            return l.conn == 8 ? launch_grid_tma_tc<LT, 8>(maps, a, l.plain, grid, st)
+                               : launch_grid_tma_tc<LT, 4>(maps, a, l.plain, grid, st);
         }
     }
     if (l.tc) {
@@ -934,10 +934,10 @@ cudaError_t launch_grid_step_lt(const GridStepLaunch &l, cudaStream_t st) {
             const cudaError_t e = encode_grid_maps(&maps, l, storage_labels(LT), GridTmaGeom<LT>::CS);
             if (e != cudaSuccess) return e;
             if (l.conn == 8)
-                return l.mu_sym ? launch_grid_tma<LT, 8, true>(maps, a, l.mu_host, grid, block, st)
-                                : launch_grid_tma<LT, 8, false>(maps, a, l.mu_host, grid, block, st);
-            return l.mu_sym ? launch_grid_tma<LT, 4, true>(maps, a, l.mu_host, grid, block, st)
-                            : launch_grid_tma<LT, 4, false>(maps, a, l.mu_host, grid, block, st);
+                return l.mu_sym ? launch_grid_tma<LT, 8, true>(maps, a, l.mu_host, l.plain, grid, block, st)
+                                : launch_grid_tma<LT, 8, false>(maps, a, l.mu_host, l.plain, grid, block, st);
+            return l.mu_sym ? launch_grid_tma<LT, 4, true>(maps, a, l.mu_host, l.plain, grid, block, st)
+                            : launch_grid_tma<LT, 4, false>(maps, a, l.mu_host, l.plain, grid, block, st);
         }
     }
     if (l.conn == 8) {

@@ -694,8 +694,8 @@ grid_tma2_step_kernel(const __grid_constant__ GridTmaMaps maps, const __grid_con
 cudaError_t encode_grid_maps(GridTmaMaps *m, const GridStepLaunch &l, int LP, int CS);
 
 template <int LT, int CONN, bool SYM>
-cudaError_t launch_grid_tma(const GridTmaMaps &maps, const GridStepArgs &a, const float2 *mu_host, dim3 grid,
-                            dim3 block, cudaStream_t st) {
+cudaError_t launch_grid_tma(const GridTmaMaps &maps, const GridStepArgs &a, const float2 *mu_host, bool plain,
+                            dim3 grid, dim3 block, cudaStream_t st) {
     constexpr int bytes = GridTmaGeom<LT>::bytes;
     static SmemOptIn optin;   // once per device
     // programmatic dependent launch: the step may start while the previous
@@ -709,7 +709,7 @@ cudaError_t launch_grid_tma(const GridTmaMaps &maps, const GridStepArgs &a, cons
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = pdl;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = plain ? 0 : 1;
     if constexpr (SYM) {
         // two pixels per thread
         auto kern = grid_tma2_step_kernel<LT, CONN>;

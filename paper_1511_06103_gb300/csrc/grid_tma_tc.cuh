@@ -468,7 +468,8 @@ grid_tma2_tc_step_kernel(const __grid_constant__ GridTmaTcMaps maps, const __gri
 cudaError_t encode_grid_tc_maps(GridTmaTcMaps *m, const GridStepLaunch &l, int LP, int CS, int C16, int UP);
 
 template <int LT, int CONN>
-cudaError_t launch_grid_tma_tc(const GridTmaTcMaps &maps, const GridStepArgs &a, dim3 grid, cudaStream_t st) {
+cudaError_t launch_grid_tma_tc(const GridTmaTcMaps &maps, const GridStepArgs &a, bool plain, dim3 grid,
+                               cudaStream_t st) {
     constexpr int bytes = GridTmaTcGeom<LT>::bytes;
     static SmemOptIn optin;   // once per device
     const cudaError_t attr = smem_optin(optin, grid_tma2_tc_step_kernel<LT, CONN>, bytes);
@@ -482,7 +483,7 @@ cudaError_t launch_grid_tma_tc(const GridTmaTcMaps &maps, const GridStepArgs &a,
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = pdl;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = plain ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, grid_tma2_tc_step_kernel<LT, CONN>, maps, a);
 }
 

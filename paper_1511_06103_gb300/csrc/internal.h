@@ -107,6 +107,9 @@ struct GridStepLaunch {
     // prev_pending = n > 0 makes this launch first sum the n partials per
     // tile of step t - 1 (trace entry, stopping rule).  0: none.
     int defer, prev_pending;
+    // The kernel launched just before may have written what a step reads ahead of its
+    // dependency wait (unaries, edge weights, mu): an ordinary launch, after all of it.
+    bool plain;
 };
 
 // Opt-in of one kernel to more than 48 KB of dynamic shared memory.  The

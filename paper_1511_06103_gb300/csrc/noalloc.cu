@@ -156,6 +156,7 @@ extern "C" crf_status mf_grid_step_noalloc(int32_t topology, int32_t n_labels, i
     a.update = 1;
     a.rel_tol = 0.0;
     a.mu_sym = sym;
+    a.plain = true;   // the set-up kernel writes mu
     if (e == cudaSuccess) e = launch_grid_step(a, st);
     if (e == cudaSuccess) {
         noalloc_finish_kernel<<<1, 1, 0, st>>>(status, F_out);
